@@ -217,7 +217,9 @@ def _prefill(case, seed):
                 ang = torch.arange(s, device="cuda", dtype=torch.float32) * (2 * math.pi / 65536)
                 k += (torch.cos(ang)[None, :, None] * _randn(g, H, 1, D)
                       + torch.sin(ang)[None, :, None] * _randn(g, H, 1, D))
-                at = torch.randint(0, s - RECENT, (H, needles), generator=g, device="cuda")
+                step = (s - RECENT) // needles   # one in every stretch, so no two at one place
+                at = torch.randint(0, step, (H, needles), generator=g, device="cuda")
+                at += step * torch.arange(needles, device="cuda")
                 k.scatter_(1, at[..., None].expand(-1, -1, D), 3 * _randn(g, H, needles, D))
             K[b] = k.to(torch.bfloat16)
             V[b] = (_randn(g, H, s, D) * vsc[:, None]).to(torch.bfloat16)
