@@ -295,7 +295,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   float *centersT = nullptr, *cnorm = nullptr, *vpart = nullptr, *oS = nullptr;
   __nv_bfloat16* cplanes = nullptr;
   double* centers64 = nullptr;
-  long long* msum = nullptr;
+  long long *msum = nullptr, *tsum = nullptr;
   uint32_t* mflag = nullptr;
   float* knorm2 = nullptr;
   int4* amb = nullptr;
@@ -324,7 +324,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
          S.get(&cnorm, size_t(UL) * rmax) && S.get(&kbar, size_t(UL) * ent_stride * kHeadDim) &&
          S.get(&vbar, size_t(UL) * ent_stride * kHeadDim) &&
          S.get(&ecount, size_t(UL) * ent_stride) &&
-         S.get(&msum, size_t(UL) * rmax * 2 * kHeadDim) && S.get(&mflag, size_t(UL) * rmax) &&
+         S.get(&msum, size_t(UL) * rmax * 2 * kHeadDim * 2) && S.get(&mflag, size_t(UL) * rmax) &&
          S.get(&knorm2, US) && S.get(&amb, US) && S.get(&amb_count, 1) &&
          S.get(&centers32, size_t(UL) * rmax * kHeadDim) && S.get(&assign2, US) &&
          S.get(&members2, US) && S.get(&cbase2, size_t(UL) * rmax) && S.get(&ccount2, size_t(UL) * rmax) &&
@@ -336,10 +336,12 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     ok = cudaMemsetAsync(assign, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
          cudaMemsetAsync(assign2, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
          cudaMemsetAsync(hist, 0, size_t(UL) * ntiles * rmax * sizeof(int32_t), stream) == cudaSuccess;
-  if (ok && rmax > 0)
-    ok = cudaMemsetAsync(msum, 0, size_t(UL) * rmax * 2 * kHeadDim * sizeof(long long), stream) ==
-             cudaSuccess &&
+  if (ok && rmax > 0) {
+    const size_t n = size_t(UL) * rmax * 2 * kHeadDim;
+    tsum = msum + n;
+    ok = cudaMemsetAsync(msum, 0, 2 * n * sizeof(long long), stream) == cudaSuccess &&
          cudaMemsetAsync(mflag, 0, size_t(UL) * rmax * sizeof(uint32_t), stream) == cudaSuccess;
+  }
   if (ok && proxy)
     ok = S.get(&vpart, size_t(UL) * n_val_rows * nchunks * kValRec) &&
          S.get(&oS, size_t(UL) * n_val_rows * kHeadDim) &&
@@ -384,6 +386,10 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
       set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_assign_tc, sm_assign) != cudaSuccess ||
       set_smem(k_lloyd_assign_pt, kPtSmemMax) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false, 0>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false, 1>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false, -1>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<true, 0>, kAccSmem) != cudaSuccess ||
       set_smem(k_val_loss, kValSmem) != cudaSuccess ||
       set_smem(k_val_full, kValSmem) != cudaSuccess)
     return cleanup_fail(fail(RESKV_ERR_CUDA, "setting kernel shared-memory limits"));
@@ -467,7 +473,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
 
     LloydArgs la{K, V, s, P, n_top, b, ntiles, rmax, top, rank_pos, nullptr, centersT, cnorm,
                  centers64, assign, hist, ccount, cbase, members, kbar, vbar, ecount,
-                 ent_stride, 0, c->status, bl_d, cplanes, msum, mflag, knorm2, amb, amb_count, centers32,
+                 ent_stride, 0, c->status, bl_d, cplanes, msum, tsum, mflag, knorm2, amb, amb_count, centers32,
                  assign2, members2, cbase2, ccount2, moved, 0};
     if (rmax > 0)
       k_key_norm2<<<unsigned(cdiv(int64_t(US), 8)), 256, 0, stream>>>(K, knorm2, int64_t(US));
@@ -518,12 +524,12 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         const dim3 ga(unsigned(cdiv(s, int64_t(kAccRows))), UL);
         if (it >= kDeltaFrom) {
           k_lloyd_moved<<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(la, int64_t(US));
-          k_lloyd_accum<false, 1><<<ga, kThreads, 0, stream>>>(la);
-          k_lloyd_accum<false, -1><<<ga, kThreads, 0, stream>>>(la);
+          k_lloyd_accum<false, 1><<<ga, kThreads, kAccSmem, stream>>>(la);
+          k_lloyd_accum<false, -1><<<ga, kThreads, kAccSmem, stream>>>(la);
         } else {
-          k_lloyd_accum<false, 0><<<ga, kThreads, 0, stream>>>(la);
+          k_lloyd_accum<false, 0><<<ga, kThreads, kAccSmem, stream>>>(la);
         }
-        if (last) k_lloyd_accum<true, 0><<<ga, kThreads, 0, stream>>>(la);
+        if (last) k_lloyd_accum<true, 0><<<ga, kThreads, kAccSmem, stream>>>(la);
         const int keep = !last && it + 1 >= kDeltaFrom;     // the next pass updates these sums
         k_lloyd_finish<<<dim3(unsigned(cdiv(int64_t(gr), kFinWarps)), UL), kFinWarps * 32, 0, stream>>>(
             la, last, keep);

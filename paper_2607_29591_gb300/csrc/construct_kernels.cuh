@@ -738,8 +738,9 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_adakv(AdaArgs p) {
 // summary; App. B: 4 iterations, initial centres = the highest-scored evicted
 // keys).  One "run" builds r_unit[ul] entries for every unit of the layer.
 // E = S \ M_r = { p < s - |P| : rank_pos[p] >= m - |P| },  m = b - r.
-// Deterministic: assignments by (distance, centre index); member sums in
-// fp64 in token order (stable counting sort); no float atomics.
+// Deterministic: assignments by (distance, centre index); exact integer member
+// sums (fp64 in token order where a value has no fixed-point form); no float
+// atomics.
 // ---------------------------------------------------------------------------
 
 constexpr int kMaxR = 8192;
@@ -773,8 +774,11 @@ struct LloydArgs {
   const int32_t* budgets;      // [UL] per-unit budgets, or NULL (budget)
   __nv_bfloat16* cplanes;      // [UL, 2, rmax, d] the fp32 centres split into
                                // two bf16 planes c1 + c2 (tensor-core operands)
-  long long* msum;             // [UL, rmax, 2, d] fixed-point member sums (K, V); zero between passes
-  uint32_t* mflag;             // [UL, rmax] set when a member value is outside the fixed-point range
+  long long* msum;             // [UL, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
+                               // 32 q + l; zero between passes
+  long long* tsum;             // [UL, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
+  uint32_t* mflag;             // [UL, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
+                               // member value is outside both
   float* knorm2;               // [UL, s] fp32 ||k||^2 of every key (the persistent assignment's bound)
   int4* amb;                   // [UL * s] tokens the persistent assignment leaves to k_lloyd_resolve
   int* amb_count;              // their number (zeroed before each assignment)
@@ -948,75 +952,121 @@ __global__ void k_lloyd_scatter(LloydArgs p) {
 
 // New centre = mean key of its members; on the last iteration also the mean
 // value, and the stored bf16 entry (Eq. summary).  The member sums are exact
-// fixed-point integers, so they are free of summation order, and the
-// conversion of the total to fp64 is the exact sum rounded once; mean = that
-// sum / count.  If a member value is outside the fixed-point range the centre
-// is summed in fp64 in member order instead.
+// integers, so they are free of summation order, and the conversion of the
+// total to fp64 is the exact sum rounded once; mean = that sum / count.
 //
 // Two kernels.  k_lloyd_accum sweeps the member list (grouped by centre)
 // token-parallel: each warp takes kAccRowsPerWarp consecutive member slots,
 // gathers their rows, keeps running sums for the centre it is in, and adds
 // them into msum[ul][j] with 64-bit integer atomics when the centre changes.
 // Integer addition is associative, so the totals do not depend on the order
-// the atomics land in.  k_lloyd_finish then forms the means, one CTA per
-// centre, and clears msum / mflag for the next pass.
+// the atomics land in.  k_lloyd_finish then forms the means, one warp per
+// centre, and clears the sums for the next pass.
 //
-// The running sums split every member value on the FP32 pipe, with two
-// magic-number roundings (no integer shifts, which would bound the kernel on
-// the integer ALU).  For |x| < 128 and x a multiple of 2^-32:
-//   s = x + C1 (C1 = 1.5 * 2^8; s lies in [256, 512), whose ulp is 2^-15),
-//   h = s - C1 (x rounded to a multiple of 2^-15; exact), l = x - h (exact,
-//   |l| <= 2^-16), t = l + C2 (C2 = 1.5 * 2^-9; t lies in [2^-9, 2^-8), ulp
-//   2^-32, so t is exact).
-// Then bits(s) - bits(C1) = h * 2^15 and bits(t) - bits(C2) = l * 2^32 as
-// integers, so a lane adds bits(s) and bits(t) into 32-bit sums (mod 2^32)
-// and the flush subtracts n * bits(C) for the n rows added: the exact
-// |sum h * 2^15| < 2^28 and |sum l * 2^32| <= 2^22 for n <= 64.  The flush
-// joins them into the 64-bit total (sum h * 2^15) * 2^17 + sum l * 2^32
-// (unit 2^-32).  A value outside the window shows as t - C2 != l (inexact:
-// a subnormal, a tail below 2^-32, inf, NaN) or as |x| >= 128; the centre is
-// then summed in fp64 instead.  Below 128 a sum of 2^17 terms stays under 2^63.
+// The running sum of a value is a pair of floats, S from C1 = 1.5 * 2^13 and T
+// from C2 = 1.5 * 2^-4, added to without error while T's grid holds the value:
+//   S' = S + x, h = S' - S, l = x - h   (Dekker's Fast2Sum, exact: |x| <= |S|)
+//   T' = T + l, g = T' - T, e = l - g   (e: what T's grid, 2^-27, drops)
+// so the sum is S + T - C1 - C2 exactly iff every e is zero.  S has to stay in
+// its binade [2^13, 2^14), which its exponent bits tell after every addition:
+// then |x| < 2^12 <= S, S is a multiple of 2^-10, |l| <= 2^-11, and T stays
+// within 64 * 2^-11 of C2 and is a multiple of 2^-27, so both convert to integers
+// of unit 2^-32.  Six packed fp32x2 additions and three ORs take two values
+// through it, where the integer form this replaces took 8 additions, 2 integer
+// additions and a maximum per value.
+// A value is dropped from when it is below 2^-20 in magnitude (about 8 in
+// 10^7 of normally distributed values, so in a few of a unit's centres): the
+// warp then adds the exact e as 64-bit integers of unit 2^-76, kept beside and
+// flushed into tsum.  Sums that leave the binade (64 rows that sum past 4096) or
+// values with bits below 2^-76 flag the centre: it is summed in fp64 in member
+// order.
 constexpr int kAccRowsPerWarp = 64;
 constexpr int kAccRows = kAccRowsPerWarp * (kThreads / 32);   // member slots per CTA
-static_assert(kAccRowsPerWarp <= 64, "the mod-2^32 lane sums must stay below 2^31");
-constexpr float kFixC1 = 384.0f;
-constexpr float kFixC2 = 0x1.8p-9f;
+constexpr float kSumC1 = 12288.0f;
+constexpr float kSumC2 = 0x1.8p-4f;
+static_assert(kAccRowsPerWarp <= 64, "T must stay within 2^-5 of C2");
+enum : uint32_t { kSumFp64 = 1u, kSumTails = 2u };            // mflag
 
-struct FixSum {
-  uint32_t hi[4], lo[4];
+struct PairSum {
+  float2 s, t;
 };
 
-struct FixState {
-  float err, mx;                 // sum of |t - C2 - l|, max |x|: exact iff 0 and < 128
+__device__ __forceinline__ PairSum pair_zero() {
+  return PairSum{make_float2(kSumC1, kSumC1), make_float2(kSumC2, kSumC2)};
+}
+
+// two values into their sums; returns what was dropped
+__device__ __forceinline__ float2 pair_add(float2 x, PairSum& a) {
+  const float2 s = fadd2(a.s, x), h = fsub2(s, a.s), l = fsub2(x, h);
+  const float2 t = fadd2(a.t, l), g = fsub2(t, a.t);
+  a.s = s;
+  a.t = t;
+  return fsub2(l, g);
+}
+
+// The fixed-point total of one sum, unit 2^-32 (exact).
+__device__ __forceinline__ long long sum_total(float s, float t) {
+  const long long c1 = 12288ll << 32, c2 = 3ll << 27;
+  return (__float2ll_rz(s * 0x1p32f) - c1) + (__float2ll_rz(t * 0x1p32f) - c2);
+}
+
+// A dropped e as an integer of unit 2^-76; exact unless it has bits below.
+__device__ __forceinline__ long long tail_units(float e, bool& ok) {
+  const float x = e * 0x1p76f;
+  const long long v = __float2ll_rz(x);
+  ok &= fabsf(x) < 0x1p62f && __ll2float_rz(v) == x;
+  return v;
+}
+
+// The lane's sums of four consecutive bf16 dims (two words, low half first).
+struct RowSum {
+  PairSum a, b;
+  long long tail[4];             // the dropped parts, unit 2^-76
+  uint32_t left;                 // OR of bits(S) ^ bits(C1)
+  bool dropped, bad;             // some lane's e was not zero; an e has bits below 2^-76
+
+  __device__ __forceinline__ void reset() {
+    a = b = pair_zero();
+    tail[0] = tail[1] = tail[2] = tail[3] = 0;
+    left = 0u;
+    dropped = bad = false;
+  }
+  // N rows, 32 words apart; every lane of the warp adds its part of them.
+  // One vote covers the N rows: where something was dropped they are taken
+  // once more for the exact e.
+  template <int N>
+  __device__ __forceinline__ void add(const uint2* w) {
+    const PairSum a0 = a, b0 = b;
+    const uint32_t c1 = __float_as_uint(kSumC1);
+    uint32_t any = 0u;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const uint2 v = w[32 * q];
+      const float2 e = pair_add(bf16x2_to_float2(v.x), a), f = pair_add(bf16x2_to_float2(v.y), b);
+      left |= (__float_as_uint(a.s.x) ^ c1) | (__float_as_uint(a.s.y) ^ c1);
+      left |= (__float_as_uint(b.s.x) ^ c1) | (__float_as_uint(b.s.y) ^ c1);
+      any |= __float_as_uint(e.x) | __float_as_uint(e.y);
+      any |= __float_as_uint(f.x) | __float_as_uint(f.y);
+    }
+    if (__any_sync(0xffffffffu, any != 0u)) {
+      dropped = true;
+      bool ok = true;
+      PairSum ta = a0, tb = b0;
+#pragma unroll 1
+      for (int q = 0; q < N; ++q) {
+        const uint2 v = w[32 * q];
+        const float2 e = pair_add(bf16x2_to_float2(v.x), ta), f = pair_add(bf16x2_to_float2(v.y), tb);
+        tail[0] += tail_units(e.x, ok);
+        tail[1] += tail_units(e.y, ok);
+        tail[2] += tail_units(f.x, ok);
+        tail[3] += tail_units(f.y, ok);
+      }
+      bad |= !ok;
+    }
+  }
+  // whether a sum left its binade (its sign or exponent bits changed)
+  __device__ __forceinline__ bool out_of_range() const { return (left & 0xff800000u) != 0u; }
 };
-
-__device__ __forceinline__ void fix_add(float x, uint32_t& hi, uint32_t& lo, FixState& st) {
-  const float s = __fadd_rn(x, kFixC1);
-  const float h = __fadd_rn(s, -kFixC1);
-  const float l = __fadd_rn(x, -h);
-  const float t = __fadd_rn(l, kFixC2);
-  st.err = __fadd_rn(st.err, fabsf(__fadd_rn(__fadd_rn(t, -kFixC2), -l)));
-  st.mx = fmaxf(st.mx, fabsf(x));
-  hi += __float_as_uint(s);
-  lo += __float_as_uint(t);
-}
-
-// four consecutive bf16 (two words, low half first) into the lane sums
-__device__ __forceinline__ void acc_row(uint2 w, FixSum& a, FixState& st) {
-  fix_add(__uint_as_float(w.x << 16), a.hi[0], a.lo[0], st);
-  fix_add(__uint_as_float(w.x & 0xffff0000u), a.hi[1], a.lo[1], st);
-  fix_add(__uint_as_float(w.y << 16), a.hi[2], a.lo[2], st);
-  fix_add(__uint_as_float(w.y & 0xffff0000u), a.hi[3], a.lo[3], st);
-}
-
-// dim q's 64-bit fixed-point total of n added rows; the lane sums are cleared
-__device__ __forceinline__ unsigned long long fix_total(FixSum& a, int q, uint32_t n) {
-  const int32_t h = int32_t(a.hi[q] - n * __float_as_uint(kFixC1));
-  const int32_t l = int32_t(a.lo[q] - n * __float_as_uint(kFixC2));
-  a.hi[q] = 0u;
-  a.lo[q] = 0u;
-  return static_cast<unsigned long long>(((long long)h << 17) + (long long)l);
-}
 
 // values = false: the key sums (every pass); values = true: the value sums
 // (the last pass), a launch of their own so each keeps 8 rows in flight per
@@ -1036,9 +1086,22 @@ __global__ void k_lloyd_moved(LloydArgs p, int64_t n_tok) {
   if ((threadIdx.x & 31) == 0 && t < n_tok) p.moved[t >> 5] = b;
 }
 
+// What bounds it: instruction issue (about 40 warp instructions per 256-byte row,
+// 2.7 issued per cycle) and DRAM, at 58 % of its rate.  A warp's rows arrive by
+// cp.async in a ring of kAccDepth batches of 8 (2 KB each), so that 8 KB per
+// warp and about 190 KB per SM are in flight whatever its registers; rows of
+// one centre are added four at a time without a look at the centre's end or at
+// what was dropped in between.  A full pass over 64 units of 32K keys (2.03 M
+// rows of 256 B, r = 51..204) takes 118 us; the integer form, whose loads went
+// through registers, took 176.
+constexpr int kAccDepth = 4;
+constexpr size_t kAccSmem = size_t(kThreads / 32) * kAccDepth * 8 * kAsgRowBytes;
+
 template <bool values, int delta>
-__global__ void __launch_bounds__(kThreads) k_lloyd_accum(LloydArgs p) {
+__global__ void __launch_bounds__(kThreads, 3) k_lloyd_accum(LloydArgs p) {
   static_assert(delta == 0 || !values, "value sums are taken in full");
+  extern __shared__ __align__(128) uint8_t acc_raw[];
+  __shared__ int2 rows_s[kThreads / 32][kAccRowsPerWarp];   // (slot, position) of the rows to add
   const int ul = blockIdx.y;
   const int r = p.r_unit[ul];
   if (r <= 0) return;
@@ -1050,96 +1113,100 @@ __global__ void __launch_bounds__(kThreads) k_lloyd_accum(LloydArgs p) {
   const int lo = blockIdx.x * kAccRows + w * kAccRowsPerWarp;
   if (lo >= n_mem) return;
   const int hi = min(n_mem, lo + kAccRowsPerWarp);
-  // the centre holding slot lo: the last j with cbase[j] <= lo (it is never
-  // empty: an empty centre shares its cbase with the next one)
+  const int32_t* mem = (delta < 0 ? p.members_prev : p.members) + int64_t(ul) * p.s;
+  const __nv_bfloat16* X = (values ? p.V : p.K) + int64_t(ul) * p.s * kHeadDim;
+  // the rows to add, in slot order: all, or those whose token moved.  A member
+  // position outside the unit only follows a failed assignment (its status is
+  // raised): row 0 is read instead of leaving the array
+  int2* rows = rows_s[w];
+  int n = 0;
+#pragma unroll
+  for (int k = 0; k < kAccRowsPerWarp / 32; ++k) {
+    const int i = lo + 32 * k + lane;
+    int pos = i < hi ? mem[i] : 0;
+    pos = uint32_t(pos) < uint32_t(p.s) ? pos : 0;
+    bool take = i < hi;
+    if constexpr (delta != 0) {
+      const int64_t t = int64_t(ul) * p.s + pos;
+      take = take && ((p.moved[t >> 5] >> (t & 31)) & 1u);
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, take);
+    if (take) rows[n + __popc(bal & ((1u << lane) - 1u))] = make_int2(i, pos);
+    n += __popc(bal);
+  }
+  if (n == 0) return;
+  __syncwarp();
+  const uint32_t ring = smem_u32(acc_raw) + uint32_t(w * kAccDepth * 8 * kAsgRowBytes);
+  const uint2* ringp = reinterpret_cast<const uint2*>(acc_raw + w * kAccDepth * 8 * kAsgRowBytes) + lane;
+  // rows 8b .. 8b + 7 into stage b % kAccDepth: half a warp per row
+  auto issue = [&](int b) {
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      const int x = 8 * b + q + (lane >> 4);
+      if (x < n)
+        cp_async16(ring + uint32_t(((b % kAccDepth) * 8 + q + (lane >> 4)) * kAsgRowBytes + (lane & 15) * 16),
+                   X + int64_t(rows[x].y) * kHeadDim + 8 * (lane & 15), 16u);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int b = 0; b < kAccDepth; ++b) issue(b);
+  // the centre holding slot rows[0]: the last j with cbase[j] <= it (it is
+  // never empty: an empty centre shares its cbase with the next one)
   int j = 0;
   for (int step = 1 << (31 - __clz(max(r - 1, 1))); step > 0; step >>= 1)
-    if (j + step < r && cb[j + step] <= lo) j += step;
+    if (j + step < r && cb[j + step] <= rows[0].x) j += step;
   int bnd = cb[j] + cc[j];
-  const int32_t* mem = (delta < 0 ? p.members_prev : p.members) + int64_t(ul) * p.s;
-  const __nv_bfloat16* Xb = (values ? p.V : p.K) + int64_t(ul) * p.s * kHeadDim + 4 * lane;
-  unsigned long long* ms = reinterpret_cast<unsigned long long*>(p.msum) +
-                           int64_t(ul) * p.rmax * 2 * kHeadDim + (values ? kHeadDim : 0) + 4 * lane;
-  FixSum sk = {};
-  FixState st = {0.0f, 0.0f};
-  uint32_t n = 0;                 // rows in the lane sums
+  const int64_t m0 = int64_t(ul) * p.rmax * 2 * kHeadDim + (values ? kHeadDim : 0) + lane;
+  unsigned long long* ms = reinterpret_cast<unsigned long long*>(p.msum) + m0;
+  unsigned long long* ts = reinterpret_cast<unsigned long long*>(p.tsum) + m0;
+  RowSum sum;
+  sum.reset();
+  int x0 = 0;                     // first of the rows in the sums
+  // the lane's sums into centre jj's totals (dim 4 lane + q at 32 q + lane, so
+  // that a warp's additions meet whole sectors)
   auto flush = [&](int jj) {
     unsigned long long* m = ms + int64_t(jj) * 2 * kHeadDim;
+    const long long v[4] = {sum_total(sum.a.s.x, sum.a.t.x), sum_total(sum.a.s.y, sum.a.t.y),
+                            sum_total(sum.b.s.x, sum.b.t.x), sum_total(sum.b.s.y, sum.b.t.y)};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const unsigned long long v = fix_total(sk, q, n);
-      atomicAdd(m + q, delta < 0 ? 0ull - v : v);
+    for (int q = 0; q < 4; ++q)
+      atomicAdd(m + 32 * q, static_cast<unsigned long long>(delta < 0 ? -v[q] : v[q]));
+    const bool bad = __any_sync(0xffffffffu, sum.bad || sum.out_of_range());
+    if (sum.dropped) {
+      unsigned long long* t = ts + int64_t(jj) * 2 * kHeadDim;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (sum.tail[q] != 0)
+          atomicAdd(t + 32 * q, static_cast<unsigned long long>(delta < 0 ? -sum.tail[q] : sum.tail[q]));
     }
-    const bool ok = st.err == 0.0f && st.mx < 128.0f;
-    if (delta >= 0 && __any_sync(0xffffffffu, !ok) && lane == 0)
-      atomicOr(p.mflag + int64_t(ul) * p.rmax + jj, 1u);
-    st = FixState{0.0f, 0.0f};
-    n = 0;
+    if ((sum.dropped || bad) && lane == 0)
+      atomicOr(p.mflag + int64_t(ul) * p.rmax + jj, (sum.dropped ? kSumTails : 0u) | (bad ? kSumFp64 : 0u));
+    sum.reset();
   };
-  for (int i32 = lo; i32 < hi; i32 += 32) {
-    // a member position outside the unit only follows a failed assignment
-    // (its status is raised): read row 0 instead of leaving the array
-    int my = i32 + lane < hi ? mem[i32 + lane] : 0;
-    my = uint32_t(my) < uint32_t(p.s) ? my : 0;
-    if constexpr (delta != 0) {
-      // the block's movers, in list order, 8 rows at a time
-      bool mv = false;
-      if (i32 + lane < hi) {
-        const int64_t t = int64_t(ul) * p.s + my;
-        mv = (p.moved[t >> 5] >> (t & 31)) & 1u;
+  for (int b = 0; 8 * b < n; ++b) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAccDepth - 1) : "memory");
+    __syncwarp();
+    const uint2* st = ringp + (b % kAccDepth) * 8 * 32 - 8 * b * 32;      // row x at st + 32 x
+    const int xe = min(n, 8 * b + 8);
+    for (int x = 8 * b; x < xe;) {
+      const int i = delta == 0 ? lo + x : rows[x].x;
+      if (i >= bnd && j < r - 1) {                // warp-uniform: row x is of a later centre
+        if (x > x0) flush(j);
+        x0 = x;
+        do {
+          ++j;
+          bnd = cb[j] + cc[j];
+        } while (i >= bnd && j < r - 1);
       }
-      unsigned take = __ballot_sync(0xffffffffu, mv);
-      while (take) {
-        int idx[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          idx[q] = take ? __ffs(take) - 1 : -1;
-          take &= take - 1;
-        }
-        uint2 kw[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int64_t pos = __shfl_sync(0xffffffffu, my, idx[q] < 0 ? 0 : idx[q]);
-          if (idx[q] >= 0) kw[q] = __ldg(reinterpret_cast<const uint2*>(Xb + pos * kHeadDim));
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (idx[q] >= 0) {
-            const int i = i32 + idx[q];
-            while (i >= bnd && j < r - 1) {   // warp-uniform: the next centre starts here
-              flush(j);
-              ++j;
-              bnd = cb[j] + cc[j];
-            }
-            acc_row(kw[q], sk, st);
-            ++n;
-          }
-        }
-      }
-    } else {
-#pragma unroll 1
-      for (int i8 = 0; i8 < 32 && i32 + i8 < hi; i8 += 8) {
-        uint2 kw[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int64_t pos = __shfl_sync(0xffffffffu, my, i8 + q);
-          if (i32 + i8 + q < hi) kw[q] = __ldg(reinterpret_cast<const uint2*>(Xb + pos * kHeadDim));
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = i32 + i8 + q;
-          if (i < hi) {
-            while (i >= bnd && j < r - 1) {   // warp-uniform: the next centre starts here
-              flush(j);
-              ++j;
-              bnd = cb[j] + cc[j];
-            }
-            acc_row(kw[q], sk, st);
-            ++n;
-          }
-        }
-      }
+      // rows of this centre: those before bnd (or the last centre's, all);
+      // movers' slots are not consecutive and are taken one by one
+      const int xs = delta != 0 ? x + 1 : (j < r - 1 ? min(xe, bnd - lo) : xe);
+      for (; x + 4 <= xs; x += 4) sum.add<4>(st + 32 * x);
+      for (; x < xs; ++x) sum.add<1>(st + 32 * x);
     }
+    __syncwarp();
+    issue(b + kAccDepth);
   }
   flush(j);
 }
@@ -1158,8 +1225,11 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   if (j >= r) return;
   const int64_t uj = int64_t(ul) * p.rmax + j;
   const int cnt = p.ccount[uj];
-  const bool exact = p.mflag[uj] == 0u;
-  long long* ms = p.msum + uj * 2 * kHeadDim + 4 * lane;
+  const uint32_t flag = p.mflag[uj];
+  const bool exact = flag == 0u;
+  // dim 4 lane + q of the key sums at 32 q, of the value sums at kHeadDim + 32 q
+  long long* ms = p.msum + uj * 2 * kHeadDim + lane;
+  long long* ts = p.tsum + uj * 2 * kHeadDim + lane;
   // mean = RN(sum / cnt) with sum = RN(S * 2^-32) for the integer sum S: by
   // Markstein's correction with the rounded reciprocal y = RN(1 / (cnt 2^32)),
   // q0 = RN(S y), r = S - q0 cnt 2^32 (exact in one fma), q = RN(q0 + r y) is
@@ -1172,15 +1242,27 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     const double bd = cd * 0x1p32;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const double sk = double(ms[q]);
+      const double sk = double(ms[32 * q]);
       const double qk = sk * y;
       mk[q] = fma(fma(-qk, bd, sk), y, qk);
       mv[q] = 0.0;
       if (final_pass) {
-        const double sv = double(ms[kHeadDim + q]);
+        const double sv = double(ms[kHeadDim + 32 * q]);
         const double qv = sv * y;
         mv[q] = fma(fma(-qv, bd, sv), y, qv);
       }
+    }
+  } else if ((flag & kSumFp64) == 0u) {
+    // some values have bits below T's grid: sum = RN(S * 2^-32 + tails * 2^-76)
+    auto total = [](long long hi, long long lo) {
+      const __int128 v = (__int128(hi) << 44) + lo;
+      const double x = v == 0 ? 0.0 : round_u128(u128(v < 0 ? -v : v), -76, false);
+      return v < 0 ? -x : x;
+    };
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      mk[q] = total(ms[32 * q], ts[32 * q]) / cd;
+      mv[q] = final_pass ? total(ms[kHeadDim + 32 * q], ts[kHeadDim + 32 * q]) / cd : 0.0;
     }
   } else {
     // fp64 sums in member order
@@ -1216,7 +1298,11 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   }
   if (!keep) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) ms[q] = ms[kHeadDim + q] = 0;
+    for (int q = 0; q < 4; ++q) ms[32 * q] = ms[kHeadDim + 32 * q] = 0;
+    if (!exact) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) ts[32 * q] = ts[kHeadDim + 32 * q] = 0;
+    }
   }
   double* c64 = p.centers64 + uj * kHeadDim + 4 * lane;
   float* c32 = p.centers32 + uj * kHeadDim + 4 * lane;
