@@ -10,8 +10,7 @@
 #include <vector>
 
 #include "construct_kernels.cuh"
-#include "lloyd_pt.cuh"
-#include "lloyd_tc.cuh"
+#include "lloyd_assign.cuh"
 #include "internal.h"
 
 namespace reskv {
@@ -245,6 +244,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   }
   for (int32_t r : col_rmax) rmax = std::max(rmax, r);
   if (rmax > kMaxR) return fail(RESKV_ERR_UNSUPPORTED, "residual entries per unit must be <= 8192");
+  const int rstride = (rmax + 15) & ~15;             // stride of the per-centre arrays
 
   // ---------------- handle and scratch ----------------
   reskv_cache* c = nullptr;
@@ -288,17 +288,19 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   float* A = nullptr;
   float2* tstats = nullptr;
   float2* rstats = nullptr;
-  int32_t *top = nullptr, *rank_pos = nullptr, *assign = nullptr, *hist = nullptr;
+  int32_t *top = nullptr, *rank_pos = nullptr, *assign = nullptr;
   int32_t *ccount = nullptr, *cbase = nullptr, *members = nullptr, *ecount = nullptr;
   int32_t *r_runs = nullptr, *r_final = nullptr, *chosen = nullptr, *run_off_d = nullptr;
   int32_t* budgets_d = nullptr;        // [U_all] per-unit budgets (per_unit only)
-  float *centersT = nullptr, *cnorm = nullptr, *vpart = nullptr, *oS = nullptr;
+  float *cnorm = nullptr, *vpart = nullptr, *oS = nullptr;
   __nv_bfloat16* cplanes = nullptr;
+  __nv_bfloat16* kpad = nullptr;       // the layer's keys where they are fewer than a tile
   double* centers64 = nullptr;
   long long *msum = nullptr, *tsum = nullptr;
   uint32_t* mflag = nullptr;
-  float* knorm2 = nullptr;
+  float* knorm = nullptr;
   int4* amb = nullptr;
+  int2* cand = nullptr;
   int* amb_count = nullptr;
   float* centers32 = nullptr;
   // the previous Lloyd iteration's assignment and member lists
@@ -316,31 +318,31 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     ok = S.get(&A, US) && S.get(&tstats, size_t(UL) * n_fit_rows * ntiles) &&
          S.get(&rstats, size_t(UL) * n_fit_rows);
   if (ok && rmax > 0)
-    ok = S.get(&assign, US) && S.get(&hist, size_t(UL) * ntiles * rmax) &&
-         S.get(&ccount, size_t(UL) * rmax) && S.get(&cbase, size_t(UL) * rmax) &&
-         S.get(&members, US) && S.get(&centersT, size_t(UL) * kHeadDim * rmax) &&
-         S.get(&centers64, size_t(UL) * kHeadDim * rmax) &&
-         S.get(&cplanes, size_t(UL) * 2 * rmax * kHeadDim) &&
-         S.get(&cnorm, size_t(UL) * rmax) && S.get(&kbar, size_t(UL) * ent_stride * kHeadDim) &&
+    ok = S.get(&assign, US) && S.get(&ccount, size_t(UL) * rstride * 2) &&
+         S.get(&cbase, size_t(UL) * rstride) && S.get(&members, US) &&
+         S.get(&centers64, size_t(UL) * kHeadDim * rstride) &&
+         S.get(&cplanes, size_t(UL) * 2 * rstride * kHeadDim) &&
+         S.get(&cnorm, size_t(UL) * rstride) && S.get(&kbar, size_t(UL) * ent_stride * kHeadDim) &&
          S.get(&vbar, size_t(UL) * ent_stride * kHeadDim) &&
          S.get(&ecount, size_t(UL) * ent_stride) &&
-         S.get(&msum, size_t(UL) * rmax * 2 * kHeadDim * 2) && S.get(&mflag, size_t(UL) * rmax) &&
-         S.get(&knorm2, US) && S.get(&amb, US) && S.get(&amb_count, 1) &&
-         S.get(&centers32, size_t(UL) * rmax * kHeadDim) && S.get(&assign2, US) &&
-         S.get(&members2, US) && S.get(&cbase2, size_t(UL) * rmax) && S.get(&ccount2, size_t(UL) * rmax) &&
-         S.get(&moved, (US + 31) / 32);
+         S.get(&msum, size_t(UL) * rstride * 2 * kHeadDim * 2) && S.get(&mflag, size_t(UL) * rstride) &&
+         S.get(&knorm, US) && S.get(&amb, size_t(UL) * ntiles * kTile) && S.get(&amb_count, kResMaxCtas) &&
+         (rmax <= kAsgRmax || S.get(&cand, US)) && (US >= size_t(kTile) || S.get(&kpad, kTile * kHeadDim)) &&
+         S.get(&centers32, size_t(UL) * rstride * kHeadDim) && S.get(&assign2, US) &&
+         S.get(&members2, US) && S.get(&cbase2, size_t(UL) * rstride) &&
+         S.get(&ccount2, size_t(UL) * rstride * 2) && S.get(&moved, (US + 31) / 32);
   // the member sums start at zero; each pass's k_lloyd_finish clears what it
-  // read.  Assignments start at -1 (no centre) and per-tile counts at 0, so
-  // that a tile a failed assignment never reached holds no index and no count
+  // read.  Assignments start at -1 (no centre), so that a tile a failed
+  // assignment never reached holds no index
   if (ok && rmax > 0)
     ok = cudaMemsetAsync(assign, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
          cudaMemsetAsync(assign2, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
-         cudaMemsetAsync(hist, 0, size_t(UL) * ntiles * rmax * sizeof(int32_t), stream) == cudaSuccess;
+         (!kpad || cudaMemsetAsync(kpad, 0, kTile * kHeadDim * 2, stream) == cudaSuccess);
   if (ok && rmax > 0) {
-    const size_t n = size_t(UL) * rmax * 2 * kHeadDim;
+    const size_t n = size_t(UL) * rstride * 2 * kHeadDim;
     tsum = msum + n;
     ok = cudaMemsetAsync(msum, 0, 2 * n * sizeof(long long), stream) == cudaSuccess &&
-         cudaMemsetAsync(mflag, 0, size_t(UL) * rmax * sizeof(uint32_t), stream) == cudaSuccess;
+         cudaMemsetAsync(mflag, 0, size_t(UL) * rstride * sizeof(uint32_t), stream) == cudaSuccess;
   }
   if (ok && proxy)
     ok = S.get(&vpart, size_t(UL) * n_val_rows * nchunks * kValRec) &&
@@ -382,10 +384,13 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   const size_t sm_obs1 = size_t(kTile) * kAsgRowBytes;               // the key tile
   const size_t sm_obs2 = sm_obs1 + size_t(kThreads / 32) * kTile * 4;  // + per-warp sums
   const size_t sm_top = size_t(kTopMax) * 12 + (256 + 32 + 4) * 4;
-  const size_t sm_assign = lloyd_tc_smem(rmax);
+  const size_t sm_scatter = size_t(std::max(rmax, 1)) * 2 * sizeof(int);
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
-      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_assign_tc, sm_assign) != cudaSuccess ||
-      set_smem(k_lloyd_assign_pt, kPtSmemMax) != cudaSuccess ||
+      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter, sm_scatter) != cudaSuccess ||
+      set_smem(k_lloyd_assign<1>, kAsgSmemMax) != cudaSuccess ||
+      set_smem(k_lloyd_assign<2>, kAsgSmemMax) != cudaSuccess ||
+      set_smem(k_lloyd_assign<3>, kAsgSmemMax) != cudaSuccess ||
+      set_smem(k_lloyd_assign<4>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_accum<false, 0>, kAccSmem) != cudaSuccess ||
       set_smem(k_lloyd_accum<false, 1>, kAccSmem) != cudaSuccess ||
       set_smem(k_lloyd_accum<false, -1>, kAccSmem) != cudaSuccess ||
@@ -471,23 +476,56 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       for (int32_t r : hr) grid_r = std::max<int>(grid_r, r);
     }
 
-    LloydArgs la{K, V, s, P, n_top, b, ntiles, rmax, top, rank_pos, nullptr, centersT, cnorm,
-                 centers64, assign, hist, ccount, cbase, members, kbar, vbar, ecount,
-                 ent_stride, 0, c->status, bl_d, cplanes, msum, tsum, mflag, knorm2, amb, amb_count, centers32,
-                 assign2, members2, cbase2, ccount2, moved, 0};
-    if (rmax > 0)
-      k_key_norm2<<<unsigned(cdiv(int64_t(US), 8)), 256, 0, stream>>>(K, knorm2, int64_t(US));
-    // the persistent assignment loads key tiles by TMA (a 16-byte aligned
-    // base and at least one whole tile of rows); otherwise the streaming form
+    LloydArgs la{};
+    la.K = K;
+    la.V = V;
+    la.s = s;
+    la.UL = la.n_units = UL;
+    la.recent = P;
+    la.n_top = n_top;
+    la.budget = b;
+    la.ntiles = ntiles;
+    la.rmax = rstride;
+    la.top = top;
+    la.rank_pos = rank_pos;
+    la.budgets = bl_d;
+    la.cnorm = cnorm;
+    la.centers64 = centers64;
+    la.centers32 = centers32;
+    la.cplanes = cplanes;
+    la.knorm = knorm;
+    la.cand = cand;
+    la.amb = amb;
+    la.amb_count = amb_count;
+    la.moved = moved;
+    la.msum = msum;
+    la.tsum = tsum;
+    la.mflag = mflag;
+    la.kbar = kbar;
+    la.vbar = vbar;
+    la.ecount = ecount;
+    la.ent_stride = ent_stride;
+    la.status = c->status;
+    // the assignment loads tiles of 128 keys by TMA: a layer with fewer rows is
+    // read from a padded copy
     CUtensorMap tmK;
-    const bool pt_keys = rmax > 0 && US >= size_t(kTile) && encode_key_tiles(&tmK, K, uint64_t(US));
+    if (rmax > 0) {
+      k_key_norm<<<unsigned(cdiv(int64_t(US), 8)), 256, 0, stream>>>(K, knorm, int64_t(US));
+      if (kpad && cudaMemcpyAsync(kpad, K, US * kHeadDim * 2, cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
+        return cleanup_fail(fail(RESKV_ERR_CUDA, "copying the keys"));
+      if (!encode_key_tiles(&tmK, kpad ? kpad : K, std::max<uint64_t>(US, kTile)))
+        return cleanup_fail(fail(RESKV_ERR_CUDA, "creating the TMA tensor map of the keys"));
+    }
     auto lloyd_run = [&](const int32_t* r_unit, int ent_off, int r_hi) -> reskv_status {
       la.r_unit = r_unit;
       la.ent_off = ent_off;
       timing_ok &= timer.mark(kStLloyd);
-      const unsigned gr = unsigned(std::max(r_hi, 1));
-      const unsigned pt_grid = unsigned(std::min<int64_t>(c->num_sms, int64_t(UL) * ntiles));
-      k_lloyd_init<<<dim3(gr, UL), kHeadDim, 0, stream>>>(la);
+      const unsigned gr = unsigned(cdiv((r_hi + 15) & ~15, kFinWarps));
+      const unsigned asg_grid = unsigned(std::min<int64_t>(std::min(c->num_sms, kResMaxCtas), int64_t(UL) * ntiles));
+      // segments of at most 256 centres, of equal width
+      const int nseg = int(cdiv(r_hi, kAsgRmax));
+      const int segw = (int(cdiv(r_hi, nseg)) + 15) & ~15;
+      k_lloyd_init<<<dim3(gr, UL), kFinWarps * 32, 0, stream>>>(la);
       // key sums in full for the first kDeltaFrom iterations, then updated
       // from the previous iteration's by the tokens that moved (a third of
       // the tokens move in the second iteration, about a tenth later)
@@ -504,22 +542,21 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         la.members_prev = prv[1];
         la.cbase_prev = prv[2];
         la.ccount_prev = prv[3];
-        if (pt_keys && r_hi <= kPtRmax) {   // the centres fit in shared memory: persistent form
-          if (cudaMemsetAsync(amb_count, 0, sizeof(int), stream) != cudaSuccess)
-            return fail(RESKV_ERR_CUDA, "clearing the ambiguous-token count");
-          const int rp = (r_hi + 15) & ~15;
-          la.test_fault = test_fault;     // an injected fault is taken by the first launch only
-          test_fault = 0;
-          k_lloyd_assign_pt<<<pt_grid, kPtThreads, lloyd_pt_smem(rp), stream>>>(la, UL, rp,
-                                                                                 lloyd_pt_key_bufs(rp), tmK);
+        la.cursor = la.ccount + size_t(UL) * rstride;
+        if (cudaMemsetAsync(la.ccount, 0, size_t(UL) * rstride * 2 * sizeof(int32_t), stream) != cudaSuccess)
+          return fail(RESKV_ERR_CUDA, "clearing the member counts");
+        la.test_fault = test_fault;       // an injected fault is taken by the first launch only
+        test_fault = 0;
+        for (int sg = 0; sg < nseg; ++sg) {
+          auto* assign_k = segw <= 64 ? k_lloyd_assign<1> : segw <= 128 ? k_lloyd_assign<2>
+                           : segw <= 192 ? k_lloyd_assign<3> : k_lloyd_assign<4>;
+          assign_k<<<asg_grid, kAsgThreads, lloyd_asg_smem(segw), stream>>>(
+              la, sg * segw, segw, lloyd_asg_key_bufs(segw), tmK);
           la.test_fault = 0;
-          k_lloyd_resolve<<<unsigned(4 * c->num_sms), kResWarps * 32, 0, stream>>>(la);
-        } else {
-          k_lloyd_assign_tc<<<dim3(ntiles, UL), kTcThreads, sm_assign, stream>>>(la);
         }
-        k_lloyd_scan<<<dim3(UL, unsigned(cdiv(int64_t(gr), kScanCentres))), kScanCentres * kScanSegs, 0, stream>>>(la);
-        k_lloyd_bases<<<UL, 256, 0, stream>>>(la);
-        k_lloyd_scatter<<<dim3(ntiles, UL), kTile, 0, stream>>>(la);
+        k_lloyd_resolve<<<unsigned(4 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
+        k_lloyd_scatter<<<dim3(unsigned(cdiv(s, int64_t(kScatterThreads))), UL), kScatterThreads,
+                          size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
         const int last = it == cfg.lloyd_iters - 1;
         const dim3 ga(unsigned(cdiv(s, int64_t(kAccRows))), UL);
         if (it >= kDeltaFrom) {
@@ -531,7 +568,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         }
         if (last) k_lloyd_accum<true, 0><<<ga, kThreads, kAccSmem, stream>>>(la);
         const int keep = !last && it + 1 >= kDeltaFrom;     // the next pass updates these sums
-        k_lloyd_finish<<<dim3(unsigned(cdiv(int64_t(gr), kFinWarps)), UL), kFinWarps * 32, 0, stream>>>(
+        k_lloyd_finish<<<dim3(unsigned(cdiv(r_hi, kFinWarps)), UL), kFinWarps * 32, 0, stream>>>(
             la, last, keep);
       }
       RESKV_LAUNCH_CHECK("residual entries");

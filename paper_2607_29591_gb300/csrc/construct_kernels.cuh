@@ -749,47 +749,50 @@ struct LloydArgs {
   const __nv_bfloat16* K;      // layer keys [UL, s, d]
   const __nv_bfloat16* V;      // layer values
   int64_t s;
+  int32_t UL;                  // (batch, KV head) units of the layer
+  int32_t n_units;             // units of this launch
   int32_t recent;              // |P| (already clamped to s)
   int32_t n_top;
   int32_t budget;
   int32_t ntiles;
-  int32_t rmax;
+  int32_t rmax;                // stride of the per-centre arrays, a multiple of 16
   const int32_t* top;          // [UL, n_top]
   const int32_t* rank_pos;     // [UL, s]
+  const int32_t* budgets;      // [UL] per-unit budgets, or NULL (budget)
   const int32_t* r_unit;       // [UL]
-  float* centersT;             // [UL, d, rmax]  fp32 copy (dim-major) for the fast path
-  float* cnorm;                // [UL, rmax]     ||c||^2 of the fp32 copy
+  float* cnorm;                // [UL, rmax]     ||c||^2 of the fp32 copy; +inf from r to the
+                               // next multiple of 16
   double* centers64;           // [UL, rmax, d]  the centres (fp64 means)
+  float* centers32;            // [UL, rmax, d]  their fp32 copy
+  __nv_bfloat16* cplanes;      // [UL, 2 planes, 2 halves, rmax, 64] the fp32 centres split into two
+                               // bf16 planes, laid out as the tensor cores read them (split_planes)
+  float* knorm;                // [UL, s] an upper bound of every key's norm (the assignment's bound)
+  int2* cand;                  // [UL, s] candidates so far (units with more than one segment)
+  int4* amb;                   // [UL * ntiles * 128] tokens the assignment leaves to k_lloyd_resolve
+  int* amb_count;              // their number, per assignment CTA
   int32_t* assign;             // [UL, s] centre index, -1 outside E
-  int32_t* hist;               // [UL, ntiles, rmax] per-tile counts, then offsets
-  int32_t* ccount;             // [UL, rmax] members per centre
+  int32_t* ccount;             // [UL, rmax] members per centre; zero before an assignment
+  int32_t* cursor;             // [UL, rmax] members placed so far; zero before an assignment
   int32_t* cbase;              // [UL, rmax] first member slot per centre
   int32_t* members;            // [UL, s] token positions grouped by centre
-  __nv_bfloat16* kbar;         // [UL, ent_stride, d] entries of this run at ent_off
-  __nv_bfloat16* vbar;
-  int32_t* ecount;             // [UL, ent_stride]
-  int64_t ent_stride;
-  int32_t ent_off;
-  uint32_t* status;
-  const int32_t* budgets;      // [UL] per-unit budgets, or NULL (budget)
-  __nv_bfloat16* cplanes;      // [UL, 2, rmax, d] the fp32 centres split into
-                               // two bf16 planes c1 + c2 (tensor-core operands)
-  long long* msum;             // [UL, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
-                               // 32 q + l; zero between passes
-  long long* tsum;             // [UL, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
-  uint32_t* mflag;             // [UL, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
-                               // member value is outside both
-  float* knorm2;               // [UL, s] fp32 ||k||^2 of every key (the persistent assignment's bound)
-  int4* amb;                   // [UL * s] tokens the persistent assignment leaves to k_lloyd_resolve
-  int* amb_count;              // their number (zeroed before each assignment)
-  float* centers32;            // [UL, rmax, d] row-major fp32 copy of the centres
   // the previous iteration's assignment and member lists (delta accumulation)
   const int32_t* assign_prev;
   const int32_t* members_prev;
   const int32_t* cbase_prev;
   const int32_t* ccount_prev;
   uint32_t* moved;             // [UL * s / 32] bit per token: its centre changed (delta accumulation)
-  int32_t test_fault;          // test hook: CTA 0's certifier gives up its first wait
+  long long* msum;             // [UL, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
+                               // 32 q + l; zero between passes
+  long long* tsum;             // [UL, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
+  uint32_t* mflag;             // [UL, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
+                               // member value is outside both
+  __nv_bfloat16* kbar;         // [UL, ent_stride, d] entries of this run at ent_off
+  __nv_bfloat16* vbar;
+  int32_t* ecount;             // [UL, ent_stride]
+  int64_t ent_stride;
+  int32_t ent_off;
+  uint32_t* status;
+  int32_t test_fault;          // test hook: CTA 0's first column wait gives up
 };
 
 __device__ __forceinline__ bool in_evicted(const LloydArgs& p, int ul, int64_t pos, int r) {
@@ -798,156 +801,104 @@ __device__ __forceinline__ bool in_evicted(const LloydArgs& p, int ul, int64_t p
   return rk >= 0 && rk >= keep;
 }
 
-// The bf16 planes of centre j, dim d: c = c1 + c2 + e, |e| <= 2^-16 |c| (the
-// remainder c - c1 is exact in fp32; each plane keeps 8 significant bits).
-__device__ __forceinline__ void write_planes(const LloydArgs& p, int ul, int j, int d, float c) {
-  const __nv_bfloat16 c1 = __float2bfloat16_rn(c);
-  const __nv_bfloat16 c2 = __float2bfloat16_rn(c - __bfloat162float(c1));
-  __nv_bfloat16* b = p.cplanes + (int64_t(ul) * 2 * p.rmax + j) * kHeadDim + d;
-  b[0] = c1;
-  b[int64_t(p.rmax) * kHeadDim] = c2;
-}
-
-// centre j = key of the (m - |P| + j)-th ranked token
-__global__ void k_lloyd_init(LloydArgs p) {
-  __shared__ float red[kHeadDim];
-  const int j = blockIdx.x, ul = blockIdx.y, d = threadIdx.x;
-  const int r = p.r_unit[ul];
-  if (j >= r) return;
-  const int32_t keep = int32_t(unit_budget(p.budgets, ul, p.budget)) - r - p.recent;
-  const int32_t pos = p.top[int64_t(ul) * p.n_top + keep + j];
-  const float c = __bfloat162float(p.K[(int64_t(ul) * p.s + pos) * kHeadDim + d]);
-  p.centersT[(int64_t(ul) * kHeadDim + d) * p.rmax + j] = c;
-  write_planes(p, ul, j, d, c);
-  p.centers64[(int64_t(ul) * p.rmax + j) * kHeadDim + d] = double(c);
-  p.centers32[(int64_t(ul) * p.rmax + j) * kHeadDim + d] = c;
-  red[d] = c * c;
-  __syncthreads();
-  if (d == 0) {
-    float n = 0.f;
-    for (int i = 0; i < kHeadDim; ++i) n += red[i];
-    p.cnorm[int64_t(ul) * p.rmax + j] = n;
+// The two bf16 planes of dims 4 lane .. 4 lane + 3 of centre j: c = c1 + c2 + e,
+// |e| <= 2^-16 |c| (the remainder c - c1 is exact in fp32; each plane keeps 8
+// significant bits).  A plane's 64-dim half is [rmax rows][128 bytes] with the
+// 16-byte chunks of a row XOR-swizzled by the row, so that a bulk copy of rows
+// is the tensor cores' K-major operand.
+__device__ __forceinline__ void split_planes(const LloydArgs& p, int u, int j, int lane, const float (&c)[4]) {
+  __nv_bfloat16 c1[4], c2[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c1[q] = __float2bfloat16_rn(c[q]);
+    c2[q] = __float2bfloat16_rn(c[q] - __bfloat162float(c1[q]));
   }
+  const int half = lane >> 4, ch = (lane & 15) >> 1;
+  uint8_t* b = reinterpret_cast<uint8_t*>(p.cplanes) + ((int64_t(u) * 4 + half) * p.rmax + j) * 128 +
+               ((ch ^ (j & 7)) << 4) + 8 * (lane & 1);
+  *reinterpret_cast<uint2*>(b) = *reinterpret_cast<const uint2*>(c1);
+  *reinterpret_cast<uint2*>(b + int64_t(p.rmax) * 256) = *reinterpret_cast<const uint2*>(c2);
 }
 
-// Lloyd assignment (k_lloyd_assign_tc, lloyd_tc.cuh): best (d0, j0), second
-// best (d1, j1) and third-best distance d2 of the centres seen so far for one
-// token; centres arrive in increasing index, so strict comparisons keep the
-// lower index on ties
-__device__ __forceinline__ void top3_insert(float& d0, int& j0, float& d1, int& j1, float& d2,
-                                            float x, int jx) {
-  const bool c0 = x < d0, c1 = x < d1, c2 = x < d2;
-  d2 = c1 ? d1 : (c2 ? x : d2);
-  d1 = c0 ? d0 : (c1 ? x : d1);
-  j1 = c0 ? j0 : (c1 ? jx : j1);
-  d0 = c0 ? x : d0;
-  j0 = c0 ? jx : j0;
-}
+constexpr int kFinWarps = 8;
 
-// Per centre: the member count of each tile becomes the tile's offset within
-// the centre's members (an exclusive prefix over tiles, in place), and the
-// total its count.  A CTA takes 32 centres of a unit; its 8 warps split the
-// tiles into 8 segments (coalesced over the 32 centres), sum them, and
-// rewrite their segment from the prefix of the segments before.
-constexpr int kScanCentres = 32;
-constexpr int kScanSegs = 8;
-
-__global__ void __launch_bounds__(kScanCentres * kScanSegs) k_lloyd_scan(LloydArgs p) {
-  __shared__ int seg[kScanSegs][kScanCentres];
-  const int ul = blockIdx.x;
-  const int r = p.r_unit[ul];
-  if (int(blockIdx.y) * kScanCentres >= r) return;
-  const int lane = threadIdx.x & 31, sg = threadIdx.x >> 5;
-  const int c = blockIdx.y * kScanCentres + lane;
-  const bool live = c < r;
-  const int T = p.ntiles, t0 = T * sg / kScanSegs, t1 = T * (sg + 1) / kScanSegs;
-  int32_t* h = p.hist + int64_t(ul) * T * p.rmax + c;
-  int sum = 0;
-  if (live) {
-    int t = t0;
-    for (; t + 16 <= t1; t += 16) {            // 16 independent loads in flight
-      int v[16];
+// centre j = key of the (m - |P| + j)-th ranked token, a warp each; the rows up
+// to the next multiple of 16 become centres no token is near
+__global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_init(LloydArgs p) {
+  const int lane = threadIdx.x & 31;
+  const int j = blockIdx.x * kFinWarps + (threadIdx.x >> 5), u = blockIdx.y, ul = u % p.UL;
+  const int r = p.r_unit[u];
+  if (j >= ((r + 15) & ~15)) return;
+  const int64_t uj = int64_t(u) * p.rmax + j;
+  float c[4] = {0.f, 0.f, 0.f, 0.f};
+  float n = INFINITY;
+  if (j < r) {
+    const int32_t keep = int32_t(unit_budget(p.budgets, ul, p.budget)) - r - p.recent;
+    const int32_t pos = p.top[int64_t(ul) * p.n_top + keep + j];
+    const uint2 w = *reinterpret_cast<const uint2*>(p.K + (int64_t(ul) * p.s + pos) * kHeadDim + 4 * lane);
+    const float2 a = bf16x2_to_float2(w.x), b = bf16x2_to_float2(w.y);
+    c[0] = a.x;
+    c[1] = a.y;
+    c[2] = b.x;
+    c[3] = b.y;
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = h[int64_t(t + u) * p.rmax];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) sum += v[u];
+    for (int q = 0; q < 4; ++q) {
+      p.centers64[uj * kHeadDim + 4 * lane + q] = double(c[q]);
+      p.centers32[uj * kHeadDim + 4 * lane + q] = c[q];
     }
-    for (; t < t1; ++t) sum += h[int64_t(t) * p.rmax];
+    n = fmaf(c[3], c[3], fmaf(c[2], c[2], fmaf(c[1], c[1], c[0] * c[0])));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
   }
-  seg[sg][lane] = sum;
-  __syncthreads();
-  int run = 0;
-  for (int k = 0; k < sg; ++k) run += seg[k][lane];
-  if (live) {
-    int t = t0;
-    for (; t + 16 <= t1; t += 16) {
-      int v[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = h[int64_t(t + u) * p.rmax];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        h[int64_t(t + u) * p.rmax] = run;
-        run += v[u];
-      }
-    }
-    for (; t < t1; ++t) {
-      const int v = h[int64_t(t) * p.rmax];
-      h[int64_t(t) * p.rmax] = run;
-      run += v;
-    }
-    if (sg == kScanSegs - 1) p.ccount[int64_t(ul) * p.rmax + c] = run;
-  }
+  split_planes(p, u, j, lane, c);
+  if (lane == 0) p.cnorm[uj] = n;
 }
 
-// Per unit: centre j's members start at cbase[j], the exclusive prefix of
-// the counts.
-__global__ void k_lloyd_bases(LloydArgs p) {
+// Evicted tokens into per-centre member lists (in any order inside a centre:
+// the member sums are integers).  A CTA takes 1024 tokens of a unit: it counts
+// them per centre in shared memory, takes each centre's place in its list with
+// one atomic, and writes the positions.  Centre j's list starts at the
+// exclusive prefix of the counts, which every CTA of the unit forms again.
+// Dynamic shared memory: 2 r ints.
+constexpr int kScatterThreads = 1024;
+
+__global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) {
+  extern __shared__ int sc_raw[];
   __shared__ int warp_sums[32];
-  const int ul = blockIdx.x;
-  const int r = p.r_unit[ul];
+  const int u = blockIdx.y;
+  const int r = p.r_unit[u];
   if (r == 0) return;
-  const int per = (r + blockDim.x - 1) / blockDim.x;      // centres per thread (contiguous)
-  const int32_t* cc = p.ccount + int64_t(ul) * p.rmax;
+  int* cnt = sc_raw;                   // the CTA's tokens per centre
+  int* at = sc_raw + r;                // where they go
+  const int64_t c0 = int64_t(u) * p.rmax;
+  const int64_t pos = int64_t(blockIdx.x) * kScatterThreads + threadIdx.x;
+  int a = pos < p.s ? p.assign[int64_t(u) * p.s + pos] : -1;
+  for (int j = threadIdx.x; j < r; j += kScatterThreads) cnt[j] = 0;
+  const int per = (r + kScatterThreads - 1) / kScatterThreads, j0 = threadIdx.x * per;
   int mine = 0;
-  for (int q = 0; q < per; ++q) {
-    const int j = threadIdx.x * per + q;
-    if (j < r) mine += cc[j];
-  }
+  for (int j = j0; j < min(j0 + per, r); ++j) mine += p.ccount[c0 + j];
   int base = block_exclusive_scan(mine, warp_sums, nullptr);
-  for (int q = 0; q < per; ++q) {
-    const int j = threadIdx.x * per + q;
-    if (j < r) {
-      p.cbase[int64_t(ul) * p.rmax + j] = base;
-      base += cc[j];
-    }
+  for (int j = j0; j < min(j0 + per, r); ++j) {
+    at[j] = base;
+    if (blockIdx.x == 0) p.cbase[c0 + j] = base;
+    base += p.ccount[c0 + j];
   }
-}
-
-// stable scatter of evicted tokens into per-centre member lists
-__global__ void k_lloyd_scatter(LloydArgs p) {
-  __shared__ int a_s[kTile];
-  const int tile = blockIdx.x, ul = blockIdx.y;
-  const int r = p.r_unit[ul];
-  if (r == 0) return;
-  const int t = threadIdx.x;
-  const int64_t pos = int64_t(tile) * kTile + t;
-  const int a = pos < p.s ? p.assign[int64_t(ul) * p.s + pos] : -1;
-  a_s[t] = a;
-  __syncthreads();
-  if (a < 0) return;
   if (a >= r) {                        // only after a failed assignment
     report_status(p.status, kStatusBadIndex);
-    return;
+    a = -1;
   }
-  int rank = 0;
-  for (int i = 0; i < t; ++i) rank += (a_s[i] == a);
-  const int64_t off = p.cbase[int64_t(ul) * p.rmax + a] +
-                      p.hist[(int64_t(ul) * p.ntiles + tile) * p.rmax + a] + rank;
+  const int rank = a >= 0 ? atomicAdd(&cnt[a], 1) : 0;
+  __syncthreads();
+  for (int j = threadIdx.x; j < r; j += kScatterThreads)
+    if (cnt[j] > 0) at[j] += atomicAdd(p.cursor + c0 + j, cnt[j]);
+  __syncthreads();
+  if (a < 0) return;
+  const int64_t off = int64_t(at[a]) + rank;
   if (off < 0 || off >= p.s) {         // counts inconsistent with the assignment: the same
     report_status(p.status, kStatusBadIndex);
     return;
   }
-  p.members[int64_t(ul) * p.s + off] = int32_t(pos);
+  p.members[int64_t(u) * p.s + off] = int32_t(pos);
 }
 
 // New centre = mean key of its members; on the last iteration also the mean
@@ -1214,8 +1165,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_lloyd_accum(LloydArgs p) {
 // One warp per centre, lane l on dims 4l..4l+3 (coalesced sums, centres and
 // entries); ||c||^2 of the fp32 centre by a butterfly (the certification
 // bounds its rounding for any summation order).
-constexpr int kFinWarps = 8;
-
 // keep: the key sums and flags stay for the next pass's update (delta
 // accumulation); otherwise both halves of the sums and the flag are cleared.
 __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, int final_pass, int keep) {
@@ -1265,29 +1214,30 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
       mv[q] = final_pass ? total(ms[kHeadDim + 32 * q], ts[kHeadDim + 32 * q]) / cd : 0.0;
     }
   } else {
-    // fp64 sums in member order
+    // fp64 sums over the unit's tokens in order
 #pragma unroll
     for (int q = 0; q < 4; ++q) tk[q] = tv[q] = 0.0;
-    const int64_t mb = p.cbase[uj];
-    const int cnt_in = (mb >= 0 && mb + cnt <= p.s) ? cnt : 0;   // see k_lloyd_accum
-    const int32_t* mem = p.members + int64_t(ul) * p.s + (cnt_in > 0 ? mb : 0);
+    const int32_t* as = p.assign + int64_t(ul) * p.s;
     const __nv_bfloat16* Kd = p.K + int64_t(ul) * p.s * kHeadDim + 4 * lane;
     const __nv_bfloat16* Vd = p.V + int64_t(ul) * p.s * kHeadDim + 4 * lane;
-    for (int i = 0; i < cnt_in; ++i) {
-      const int64_t pos = uint32_t(mem[i]) < uint32_t(p.s) ? mem[i] : 0;   // see k_lloyd_accum
-      const uint2 kw = *reinterpret_cast<const uint2*>(Kd + pos * kHeadDim);
-      const float2 k01 = bf16x2_to_float2(kw.x), k23 = bf16x2_to_float2(kw.y);
-      tk[0] += double(k01.x);
-      tk[1] += double(k01.y);
-      tk[2] += double(k23.x);
-      tk[3] += double(k23.y);
-      if (final_pass) {
-        const uint2 vw = *reinterpret_cast<const uint2*>(Vd + pos * kHeadDim);
-        const float2 v01 = bf16x2_to_float2(vw.x), v23 = bf16x2_to_float2(vw.y);
-        tv[0] += double(v01.x);
-        tv[1] += double(v01.y);
-        tv[2] += double(v23.x);
-        tv[3] += double(v23.y);
+    for (int64_t t0 = 0; t0 < p.s; t0 += 32) {
+      unsigned take = __ballot_sync(0xffffffffu, t0 + lane < p.s && as[t0 + lane] == j);
+      for (; take != 0u; take &= take - 1) {
+        const int64_t pos = t0 + __ffs(take) - 1;
+        const uint2 kw = *reinterpret_cast<const uint2*>(Kd + pos * kHeadDim);
+        const float2 k01 = bf16x2_to_float2(kw.x), k23 = bf16x2_to_float2(kw.y);
+        tk[0] += double(k01.x);
+        tk[1] += double(k01.y);
+        tk[2] += double(k23.x);
+        tk[3] += double(k23.y);
+        if (final_pass) {
+          const uint2 vw = *reinterpret_cast<const uint2*>(Vd + pos * kHeadDim);
+          const float2 v01 = bf16x2_to_float2(vw.x), v23 = bf16x2_to_float2(vw.y);
+          tv[0] += double(v01.x);
+          tv[1] += double(v01.y);
+          tv[2] += double(v23.x);
+          tv[3] += double(v23.y);
+        }
       }
     }
 #pragma unroll
@@ -1310,13 +1260,11 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   if (cnt > 0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int d = 4 * lane + q;
       cf[q] = float(mk[q]);
       c64[q] = mk[q];
       c32[q] = cf[q];
-      p.centersT[(int64_t(ul) * kHeadDim + d) * p.rmax + j] = cf[q];
-      write_planes(p, ul, j, d, cf[q]);
     }
+    split_planes(p, ul, j, lane, cf);
   } else {                            // an empty centre keeps its place
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
