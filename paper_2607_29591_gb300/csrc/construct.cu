@@ -77,6 +77,26 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// One cluster of CTAs of kTopThreads threads per item: as many CTAs as the SMs
+// hold (a power of two, at most 8).
+template <typename Kernel, typename Args>
+cudaError_t launch_clusters(Kernel kernel, int items, int num_sms, size_t smem, cudaStream_t stream, const Args& args) {
+  int cs = 8;
+  while (cs > 1 && int64_t(items) * cs > num_sms) cs /= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(items) * unsigned(cs), 1, 1);
+  cfg.blockDim = dim3(kTopThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = unsigned(cs);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 // Device time per construction stage: an event is recorded on the stream at
 // every stage boundary of a layer; at the end of the layer the intervals are
 // added to their stages (events are reused from layer to layer).
@@ -308,6 +328,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   int32_t *ccount = nullptr, *cbase = nullptr, *members = nullptr, *ecount = nullptr;
   int32_t *r_runs = nullptr, *r_final = nullptr, *chosen = nullptr, *run_off_d = nullptr;
   int32_t* budgets_d = nullptr;        // [U_all] per-unit budgets (per_unit only)
+  int32_t* ada_counts = nullptr;       // [UL, 2]
   float *cnorm = nullptr, *vpart = nullptr, *oS = nullptr;
   __nv_bfloat16* cplanes = nullptr;
   __nv_bfloat16* kpad = nullptr;       // the layer's keys where they are fewer than a tile
@@ -334,6 +355,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   S.get(&chosen, UL);
   S.get(&run_off_d, run_off.size());
   if (per_unit) S.get(&budgets_d, size_t(U_all));
+  if (adakv) S.get(&ada_counts, size_t(UL) * 2);
   if (n_fit_rows > 0) {
     S.get(&A, US);
     S.get(&tstats, size_t(UL) * n_fit_rows * ntiles);
@@ -420,7 +442,10 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   // kernel attributes
   const size_t sm_obs1 = size_t(kTile) * kAsgRowBytes;               // the key tile
   const size_t sm_obs2 = sm_obs1 + size_t(kThreads / 32) * kTile * 4;  // + per-warp sums
-  const size_t sm_top = size_t(kTopMax) * 12 + (256 + 32 + 4) * 4;
+  // the ranked keys and positions, up to the next power of two of kTopThreads
+  size_t n_sort = kTopThreads;
+  while (n_sort < size_t(std::max(n_top, 1))) n_sort *= 2;
+  const size_t sm_top = n_sort * 12;
   const size_t sm_scatter = size_t(std::max(rmax, 1)) * 2 * sizeof(int);
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
       set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter, sm_scatter) != cudaSuccess ||
@@ -464,10 +489,12 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     if (adakv) {
       // AdaKV: mark every head's safeguard (its top f), split the shared slots
       TopArgs tf{scores, s, P, ada_f, top, rank_pos, c->status, nullptr};
-      k_topk<<<UL, kTopThreads, sm_top, stream>>>(tf);
+      const cudaError_t e1 = launch_clusters(k_topk, UL, c->num_sms, sm_top, stream, tf);
       AdaArgs aa{scores, rank_pos, s, P, cfg.n_kv_heads, ada_f, P + ada_f,
-                 int64_t(cfg.n_kv_heads) * (n_free_head - ada_f), bl_d};
-      k_adakv<<<cfg.batch, kTopThreads, 0, stream>>>(aa);
+                 int64_t(cfg.n_kv_heads) * (n_free_head - ada_f), bl_d, ada_counts};
+      const cudaError_t e2 = launch_clusters(k_adakv, cfg.batch, c->num_sms, 0, stream, aa);
+      if (e1 != cudaSuccess || e2 != cudaSuccess)
+        return cleanup_fail(fail(RESKV_ERR_CUDA, "launching the AdaKV budgets"));
       RESKV_LAUNCH_CHECK("AdaKV budgets");
       if (cudaMemcpyAsync(budgets_host.data() + size_t(l) * UL, bl_d, size_t(UL) * 4,
                           cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
@@ -497,7 +524,8 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         cudaMemsetAsync(top, 0xff, size_t(UL) * n_top * 4, stream) != cudaSuccess)
       return cleanup_fail(fail(RESKV_ERR_CUDA, "clearing the ranking"));
     TopArgs ta{scores, s, P, n_top, top, rank_pos, c->status, bl_d};
-    k_topk<<<UL, kTopThreads, sm_top, stream>>>(ta);
+    if (launch_clusters(k_topk, UL, c->num_sms, sm_top, stream, ta) != cudaSuccess)
+      return cleanup_fail(fail(RESKV_ERR_CUDA, "launching the ranking"));
     RESKV_LAUNCH_CHECK("ranking");
     // candidate r per unit of this layer
     int grid_r = rmax;
