@@ -325,7 +325,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   float2* tstats = nullptr;
   float2* rstats = nullptr;
   int32_t *top = nullptr, *rank_pos = nullptr, *assign = nullptr;
-  int32_t *ccount = nullptr, *cbase = nullptr, *members = nullptr, *ecount = nullptr;
+  int32_t *ccount = nullptr, *ecount = nullptr;
   int32_t *r_runs = nullptr, *r_final = nullptr, *chosen = nullptr, *run_off_d = nullptr;
   int32_t* budgets_d = nullptr;        // [U_all] per-unit budgets (per_unit only)
   int32_t* ada_counts = nullptr;       // [UL, 2]
@@ -340,13 +340,19 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   int2* cand = nullptr;
   int* amb_count = nullptr;
   float* centers32 = nullptr;
-  // the previous Lloyd iteration's assignment and member lists
-  int32_t *assign2 = nullptr, *members2 = nullptr, *cbase2 = nullptr, *ccount2 = nullptr;
-  uint32_t* moved = nullptr;
+  int32_t *assign2 = nullptr, *lbase = nullptr, *lsize = nullptr, *list = nullptr, *mcount = nullptr;
   __nv_bfloat16 *kbar = nullptr, *vbar = nullptr;
   double *rowerr = nullptr, *losses = nullptr;
   const size_t US = size_t(UL) * size_t(s);
   const int nruns = proxy ? ncol : 2;
+  // Candidates whose Lloyd runs share their launches: a layer of few tokens does
+  // not fill the GPU with one (8 units of 32K keys: 1.45 ms one by one, 0.78
+  // together), one of more than 2^20 tokens does, and would pay for its small
+  // candidates being swept like the largest.
+  const int n_cands = proxy ? ncol - 1 : 1;
+  const int n_batch = int(std::max<int64_t>(
+      1, std::min({int64_t(n_cands), (int64_t(1) << 20) / int64_t(US), int64_t(65535) / UL})));   // (a grid dimension)
+  const size_t UR = size_t(UL) * n_batch;          // run units of a launch
   S.get(&scores, US);
   S.get(&top, size_t(UL) * std::max(n_top, 1));
   S.get(&rank_pos, US);
@@ -362,16 +368,14 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     S.get(&rstats, size_t(UL) * n_fit_rows);
   }
   if (rmax > 0) {
-    const size_t n_c = size_t(UL) * rstride;         // centres
-    S.get(&assign, US);
-    S.get(&assign2, US);
-    S.get(&members, US);
-    S.get(&members2, US);
-    S.get(&ccount, n_c * 2);
-    S.get(&ccount2, n_c * 2);
-    S.get(&cbase, n_c);
-    S.get(&cbase2, n_c);
-    S.get(&moved, (US + 31) / 32);
+    const size_t n_c = UR * rstride;                 // centres
+    S.get(&assign, UR * s);
+    S.get(&assign2, UR * s);
+    S.get(&list, 2 * UR * s);
+    S.get(&mcount, n_c * 2 * 2);
+    S.get(&lbase, n_c * 2);
+    S.get(&lsize, UR);
+    S.get(&ccount, n_c);
     S.get(&centers64, n_c * kHeadDim);
     S.get(&centers32, n_c * kHeadDim);
     S.get(&cplanes, n_c * 2 * kHeadDim);
@@ -382,9 +386,9 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     S.get(&msum, n_c * 2 * kHeadDim * 2);
     S.get(&mflag, n_c);
     S.get(&knorm, US);
-    S.get(&amb, size_t(UL) * ntiles * kTile);
+    S.get(&amb, UR * ntiles * kTile);
     S.get(&amb_count, kResMaxCtas);
-    if (rmax > kAsgRmax) S.get(&cand, US);
+    if (rmax > kAsgRmax) S.get(&cand, UR * s);
     if (US < size_t(kTile)) S.get(&kpad, kTile * kHeadDim);
   }
   if (proxy) {
@@ -398,14 +402,14 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   // read.  Assignments start at -1 (no centre), so that a tile a failed
   // assignment never reached holds no index
   if (ok && rmax > 0)
-    ok = cudaMemsetAsync(assign, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
-         cudaMemsetAsync(assign2, 0xff, US * sizeof(int32_t), stream) == cudaSuccess &&
+    ok = cudaMemsetAsync(assign, 0xff, UR * s * sizeof(int32_t), stream) == cudaSuccess &&
+         cudaMemsetAsync(assign2, 0xff, UR * s * sizeof(int32_t), stream) == cudaSuccess &&
          (!kpad || cudaMemsetAsync(kpad, 0, kTile * kHeadDim * 2, stream) == cudaSuccess);
   if (ok && rmax > 0) {
-    const size_t n = size_t(UL) * rstride * 2 * kHeadDim;
+    const size_t n = UR * rstride * 2 * kHeadDim;
     tsum = msum + n;
     ok = cudaMemsetAsync(msum, 0, 2 * n * sizeof(long long), stream) == cudaSuccess &&
-         cudaMemsetAsync(mflag, 0, size_t(UL) * rstride * sizeof(uint32_t), stream) == cudaSuccess;
+         cudaMemsetAsync(mflag, 0, UR * rstride * sizeof(uint32_t), stream) == cudaSuccess;
   }
   if (ok && cfg.keep_debug) {
     const size_t U = size_t(c->n_units);
@@ -446,17 +450,16 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   size_t n_sort = kTopThreads;
   while (n_sort < size_t(std::max(n_top, 1))) n_sort *= 2;
   const size_t sm_top = n_sort * 12;
-  const size_t sm_scatter = size_t(std::max(rmax, 1)) * 2 * sizeof(int);
+  const size_t sm_scatter = size_t(std::max(rmax, 1)) * 4 * sizeof(int);
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
-      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter, sm_scatter) != cudaSuccess ||
+      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false>, sm_scatter) != cudaSuccess ||
+      set_smem(k_lloyd_scatter<true>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_assign<1>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<2>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<3>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<4>, kAsgSmemMax) != cudaSuccess ||
-      set_smem(k_lloyd_accum<false, 0>, kAccSmem) != cudaSuccess ||
-      set_smem(k_lloyd_accum<false, 1>, kAccSmem) != cudaSuccess ||
-      set_smem(k_lloyd_accum<false, -1>, kAccSmem) != cudaSuccess ||
-      set_smem(k_lloyd_accum<true, 0>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<true>, kAccSmem) != cudaSuccess ||
       set_smem(k_val_loss, kValSmem) != cudaSuccess ||
       set_smem(k_val_full, kValSmem) != cudaSuccess)
     return cleanup_fail(fail(RESKV_ERR_CUDA, "setting kernel shared-memory limits"));
@@ -545,7 +548,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     la.K = K;
     la.V = V;
     la.s = s;
-    la.UL = la.n_units = UL;
+    la.UL = UL;
     la.recent = P;
     la.n_top = n_top;
     la.budget = b;
@@ -562,7 +565,12 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     la.cand = cand;
     la.amb = amb;
     la.amb_count = amb_count;
-    la.moved = moved;
+    la.mcount = mcount;
+    la.cursor = mcount + 2 * UR * rstride;
+    la.ccount = ccount;
+    la.lbase = lbase;
+    la.lsize = lsize;
+    la.list = list;
     la.msum = msum;
     la.tsum = tsum;
     la.mflag = mflag;
@@ -581,35 +589,31 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       if (!encode_key_tiles(&tmK, kpad ? kpad : K, std::max<uint64_t>(US, kTile)))
         return cleanup_fail(fail(RESKV_ERR_CUDA, "creating the TMA tensor map of the keys"));
     }
-    auto lloyd_run = [&](const int32_t* r_unit, int ent_off, int r_hi) -> reskv_status {
+    // the Lloyd runs of n_run candidates at once: r_unit [n_run, UL], entries at
+    // run_off_d[run0 ..]
+    auto lloyd_run = [&](const int32_t* r_unit, int run0, int n_run, int r_hi) -> reskv_status {
+      const int U = UL * n_run;
       la.r_unit = r_unit;
-      la.ent_off = ent_off;
+      la.n_units = U;
+      la.run_off = run_off_d + run0;
       timing_ok &= timer.mark(kStLloyd);
       const unsigned gr = unsigned(cdiv((r_hi + 15) & ~15, kFinWarps));
-      const unsigned asg_grid = unsigned(std::min<int64_t>(std::min(c->num_sms, kResMaxCtas), int64_t(UL) * ntiles));
+      const unsigned asg_grid = unsigned(std::min<int64_t>(std::min(c->num_sms, kResMaxCtas), int64_t(U) * ntiles));
       // segments of at most 256 centres, of equal width
       const int nseg = int(cdiv(r_hi, kAsgRmax));
       const int segw = (int(cdiv(r_hi, nseg)) + 15) & ~15;
-      k_lloyd_init<<<dim3(gr, UL), kFinWarps * 32, 0, stream>>>(la);
-      // key sums in full for the first kDeltaFrom iterations, then updated
-      // from the previous iteration's by the tokens that moved (a third of
-      // the tokens move in the second iteration, about a tenth later)
-      constexpr int kDeltaFrom = 2;
-      int32_t* const abuf[2][4] = {{assign, members, cbase, ccount}, {assign2, members2, cbase2, ccount2}};
+      const dim3 gs(unsigned(cdiv(s, int64_t(kScatterThreads))), unsigned(U));
+      const dim3 ga(unsigned(cdiv(s, int64_t(kAccRows))), unsigned(U));
+      auto clear = [&](int32_t* counts, size_t n) {
+        return cudaMemsetAsync(counts, 0, n * sizeof(int32_t), stream) == cudaSuccess;
+      };
+      k_lloyd_init<<<dim3(gr, U), kFinWarps * 32, 0, stream>>>(la);
       for (int it = 0; it < cfg.lloyd_iters; ++it) {
-        int32_t* const* cur = abuf[it & 1];
-        int32_t* const* prv = abuf[(it + 1) & 1];
-        la.assign = cur[0];
-        la.members = cur[1];
-        la.cbase = cur[2];
-        la.ccount = cur[3];
-        la.assign_prev = prv[0];
-        la.members_prev = prv[1];
-        la.cbase_prev = prv[2];
-        la.ccount_prev = prv[3];
-        la.cursor = la.ccount + size_t(UL) * rstride;
-        if (cudaMemsetAsync(la.ccount, 0, size_t(UL) * rstride * 2 * sizeof(int32_t), stream) != cudaSuccess)
-          return fail(RESKV_ERR_CUDA, "clearing the member counts");
+        const bool last = it == cfg.lloyd_iters - 1;
+        la.assign = (it & 1) ? assign2 : assign;
+        la.assign_prev = it == 0 ? nullptr : (it & 1) ? assign : assign2;
+        if (!clear(la.mcount, UR * rstride * 2 * 2))      // and the cursors
+          return fail(RESKV_ERR_CUDA, "clearing the move counts");
         la.test_fault = test_fault;       // an injected fault is taken by the first launch only
         test_fault = 0;
         for (int sg = 0; sg < nseg; ++sg) {
@@ -620,21 +624,17 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
           la.test_fault = 0;
         }
         k_lloyd_resolve<<<unsigned(4 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
-        k_lloyd_scatter<<<dim3(unsigned(cdiv(s, int64_t(kScatterThreads))), UL), kScatterThreads,
-                          size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
-        const int last = it == cfg.lloyd_iters - 1;
-        const dim3 ga(unsigned(cdiv(s, int64_t(kAccRows))), UL);
-        if (it >= kDeltaFrom) {
-          k_lloyd_moved<<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(la, int64_t(US));
-          k_lloyd_accum<false, 1><<<ga, kThreads, kAccSmem, stream>>>(la);
-          k_lloyd_accum<false, -1><<<ga, kThreads, kAccSmem, stream>>>(la);
-        } else {
-          k_lloyd_accum<false, 0><<<ga, kThreads, kAccSmem, stream>>>(la);
+        k_lloyd_scatter<false><<<gs, kScatterThreads, size_t(r_hi) * 4 * sizeof(int), stream>>>(la);
+        k_lloyd_accum<false><<<ga, kThreads, kAccSmem, stream>>>(la);
+        if (last) {                       // the values of every member
+          if (it > 0) {
+            if (!clear(la.cursor, UR * rstride * 2))
+              return fail(RESKV_ERR_CUDA, "clearing the list cursors");
+            k_lloyd_scatter<true><<<gs, kScatterThreads, size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
+          }
+          k_lloyd_accum<true><<<ga, kThreads, kAccSmem, stream>>>(la);
         }
-        if (last) k_lloyd_accum<true, 0><<<ga, kThreads, kAccSmem, stream>>>(la);
-        const int keep = !last && it + 1 >= kDeltaFrom;     // the next pass updates these sums
-        k_lloyd_finish<<<dim3(unsigned(cdiv(r_hi, kFinWarps)), UL), kFinWarps * 32, 0, stream>>>(
-            la, last, keep);
+        k_lloyd_finish<<<dim3(unsigned(cdiv(r_hi, kFinWarps)), U), kFinWarps * 32, 0, stream>>>(la, last);
       }
       RESKV_LAUNCH_CHECK("residual entries");
       return RESKV_OK;
@@ -649,17 +649,22 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       RESKV_LAUNCH_CHECK("validation targets");
       for (int run = 0; run < ncol; ++run) {
         const int32_t* r_unit = r_runs + size_t(run) * UL;
-        if (run > 0) {
+        auto r_most = [&](int k) {       // the largest r of candidate k (0: no unit has it)
           int r_hi = 0;
-          for (int i = 0; i < UL; ++i) r_hi = std::max(r_hi, hr[size_t(run) * UL + i]);
-          if (r_hi == 0) {           // no unit of the layer has this candidate
-            k_loss_reduce<<<unsigned(cdiv(UL, 128)), 128, 0, stream>>>(rowerr, losses, 0, UL,
-                                                                      ncol, run, r_unit);
-            RESKV_LAUNCH_CHECK("validation loss");
-            continue;
-          }
-          st = lloyd_run(r_unit, run_off[run], r_hi);
-          if (st != RESKV_OK) return cleanup_fail(st);
+          for (int i = 0; i < UL; ++i) r_hi = std::max(r_hi, hr[size_t(k) * UL + i]);
+          return r_hi;
+        };
+        if (run > 0 && (run - 1) % n_batch == 0) {
+          const int n_run = std::min(n_batch, ncol - run);
+          int r_hi = 0;
+          for (int k = run; k < run + n_run; ++k) r_hi = std::max(r_hi, r_most(k));
+          if (r_hi > 0 && (st = lloyd_run(r_unit, run, n_run, r_hi)) != RESKV_OK) return cleanup_fail(st);
+        }
+        if (run > 0 && r_most(run) == 0) {
+          k_loss_reduce<<<unsigned(cdiv(UL, 128)), 128, 0, stream>>>(rowerr, losses, 0, UL,
+                                                                    ncol, run, r_unit);
+          RESKV_LAUNCH_CHECK("validation loss");
+          continue;
         }
         timing_ok &= timer.mark(kStValLoss);
         LossArgs lo{K, V, Q, s, G, cfg.n_obs, cfg.n_val, n_val_rows, P, n_top, b, top, r_unit,
@@ -690,7 +695,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
           cudaStreamSynchronize(stream) != cudaSuccess)
         return cleanup_fail(fail(RESKV_ERR_CUDA, "copying residual counts"));
       if (any) {
-        st = lloyd_run(r_final, 0, *std::max_element(rl.begin(), rl.end()));
+        st = lloyd_run(r_final, 0, 1, *std::max_element(rl.begin(), rl.end()));
         if (st != RESKV_OK) return cleanup_fail(st);
       }
     }

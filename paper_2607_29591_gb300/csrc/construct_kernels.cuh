@@ -854,12 +854,14 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_adakv(AdaArgs p) {
 
 constexpr int kMaxR = 8192;
 
+// A launch works on n_units "runs of a unit": run unit u is unit u % UL of the
+// layer, with candidate u / UL of the launch's.
 struct LloydArgs {
   const __nv_bfloat16* K;      // layer keys [UL, s, d]
   const __nv_bfloat16* V;      // layer values
   int64_t s;
   int32_t UL;                  // (batch, KV head) units of the layer
-  int32_t n_units;             // units of this launch
+  int32_t n_units;             // run units of this launch (U below)
   int32_t recent;              // |P| (already clamped to s)
   int32_t n_top;
   int32_t budget;
@@ -868,47 +870,40 @@ struct LloydArgs {
   const int32_t* top;          // [UL, n_top]
   const int32_t* rank_pos;     // [UL, s]
   const int32_t* budgets;      // [UL] per-unit budgets, or NULL (budget)
-  const int32_t* r_unit;       // [UL]
-  float* cnorm;                // [UL, rmax]     ||c||^2 of the fp32 copy; +inf from r to the
+  const int32_t* r_unit;       // [U]
+  float* cnorm;                // [U, rmax]     ||c||^2 of the fp32 copy; +inf from r to the
                                // next multiple of 16
-  double* centers64;           // [UL, rmax, d]  the centres (fp64 means)
-  float* centers32;            // [UL, rmax, d]  their fp32 copy
-  __nv_bfloat16* cplanes;      // [UL, 2 planes, 2 halves, rmax, 64] the fp32 centres split into two
+  double* centers64;           // [U, rmax, d]  the centres (fp64 means)
+  float* centers32;            // [U, rmax, d]  their fp32 copy
+  __nv_bfloat16* cplanes;      // [U, 2 planes, 2 halves, rmax, 64] the fp32 centres split into two
                                // bf16 planes, laid out as the tensor cores read them (split_planes)
   float* knorm;                // [UL, s] an upper bound of every key's norm (the assignment's bound)
-  int2* cand;                  // [UL, s] candidates so far (units with more than one segment)
-  int4* amb;                   // [UL * ntiles * 128] tokens the assignment leaves to k_lloyd_resolve
+  int2* cand;                  // [U, s] candidates so far (units with more than one segment)
+  int4* amb;                   // [U * ntiles * 128] tokens the assignment leaves to k_lloyd_resolve
   int* amb_count;              // their number, per assignment CTA
-  int32_t* assign;             // [UL, s] centre index, -1 outside E
-  int32_t* ccount;             // [UL, rmax] members per centre; zero before an assignment
-  int32_t* cursor;             // [UL, rmax] members placed so far; zero before an assignment
-  int32_t* cbase;              // [UL, rmax] first member slot per centre
-  int32_t* members;            // [UL, s] token positions grouped by centre
-  // the previous iteration's assignment and member lists (delta accumulation)
-  const int32_t* assign_prev;
-  const int32_t* members_prev;
-  const int32_t* cbase_prev;
-  const int32_t* ccount_prev;
-  uint32_t* moved;             // [UL * s / 32] bit per token: its centre changed (delta accumulation)
-  long long* msum;             // [UL, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
-                               // 32 q + l; zero between passes
-  long long* tsum;             // [UL, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
-  uint32_t* mflag;             // [UL, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
+  int32_t* assign;             // [U, s] centre index, -1 outside E
+  const int32_t* assign_prev;  // the iteration before, or NULL in the first (no token has a centre)
+  int32_t* mcount;             // [U, 2, rmax] tokens that joined and that left a centre; zero before
+                               // an assignment
+  int32_t* cursor;             // [U, 2, rmax] of these, placed so far; zero before an assignment
+  int32_t* ccount;             // [U, rmax] members per centre before this iteration
+  int32_t* lbase;              // [U, 2, rmax] first list slot per group
+  int32_t* lsize;              // [U] slots of the list
+  int32_t* list;               // [U, 2 s] token positions: those that joined, grouped by centre, then
+                               // those that left, grouped by centre (or every member, by centre)
+  long long* msum;             // [U, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
+                               // 32 q + l; zero between runs
+  long long* tsum;             // [U, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
+  uint32_t* mflag;             // [U, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
                                // member value is outside both
-  __nv_bfloat16* kbar;         // [UL, ent_stride, d] entries of this run at ent_off
+  __nv_bfloat16* kbar;         // [UL, ent_stride, d] entries, candidate c's at run_off[c]
   __nv_bfloat16* vbar;
   int32_t* ecount;             // [UL, ent_stride]
   int64_t ent_stride;
-  int32_t ent_off;
+  const int32_t* run_off;      // [candidates of the launch]
   uint32_t* status;
   int32_t test_fault;          // test hook: CTA 0's first column wait gives up
 };
-
-__device__ __forceinline__ bool in_evicted(const LloydArgs& p, int ul, int64_t pos, int r) {
-  const int32_t rk = p.rank_pos[int64_t(ul) * p.s + pos];
-  const int32_t keep = int32_t(unit_budget(p.budgets, ul, p.budget)) - r - p.recent;  // ranked main
-  return rk >= 0 && rk >= keep;
-}
 
 // The two bf16 planes of dims 4 lane .. 4 lane + 3 of centre j: c = c1 + c2 + e,
 // |e| <= 2^-16 |c| (the remainder c - c1 is exact in fp32; each plane keeps 8
@@ -963,51 +958,73 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_init(LloydArgs p) {
   if (lane == 0) p.cnorm[uj] = n;
 }
 
-// Evicted tokens into per-centre member lists (in any order inside a centre:
-// the member sums are integers).  A CTA takes 1024 tokens of a unit: it counts
-// them per centre in shared memory, takes each centre's place in its list with
-// one atomic, and writes the positions.  Centre j's list starts at the
-// exclusive prefix of the counts, which every CTA of the unit forms again.
-// Dynamic shared memory: 2 r ints.
+// Tokens into lists grouped by centre (in any order inside a group: the member
+// sums are integers).  kMembers = false: the tokens whose centre changed in this
+// iteration, once by the centre they joined and once by the one they left (in the
+// first iteration every evicted token joins); kMembers = true: every member by
+// its centre.  A CTA takes 1024 tokens of a unit: it counts them per group in
+// shared memory, takes each group's place in its list with one atomic, and
+// writes the positions.  The groups start at the exclusive prefix of their
+// sizes, which every CTA of the unit forms again.  Dynamic shared memory: 4 r
+// ints.
 constexpr int kScatterThreads = 1024;
 
+template <bool kMembers>
 __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) {
   extern __shared__ int sc_raw[];
   __shared__ int warp_sums[32];
   const int u = blockIdx.y;
   const int r = p.r_unit[u];
   if (r == 0) return;
-  int* cnt = sc_raw;                   // the CTA's tokens per centre
-  int* at = sc_raw + r;                // where they go
+  const int ng = kMembers ? r : 2 * r;       // groups
+  int* cnt = sc_raw;                         // the CTA's tokens per group
+  int* at = sc_raw + ng;                     // where they go
   const int64_t c0 = int64_t(u) * p.rmax;
+  // size of group g, and its place in the [2, rmax] arrays
+  auto slot = [&](int g) { return 2 * c0 + (g < r ? g : p.rmax + g - r); };
+  auto size = [&](int g) {
+    if constexpr (!kMembers) return p.mcount[slot(g)];
+    else
+      return (p.assign_prev ? p.ccount[c0 + g] : 0) + p.mcount[2 * c0 + g] - p.mcount[2 * c0 + p.rmax + g];
+  };
   const int64_t pos = int64_t(blockIdx.x) * kScatterThreads + threadIdx.x;
-  int a = pos < p.s ? p.assign[int64_t(u) * p.s + pos] : -1;
-  for (int j = threadIdx.x; j < r; j += kScatterThreads) cnt[j] = 0;
-  const int per = (r + kScatterThreads - 1) / kScatterThreads, j0 = threadIdx.x * per;
+  int a = -1, o = -1;                        // the token's centre now and before
+  if (pos < p.s) {
+    a = p.assign[int64_t(u) * p.s + pos];
+    if (!kMembers && p.assign_prev) o = p.assign_prev[int64_t(u) * p.s + pos];
+  }
+  for (int g = threadIdx.x; g < ng; g += kScatterThreads) cnt[g] = 0;
+  const int per = (ng + kScatterThreads - 1) / kScatterThreads, g0 = threadIdx.x * per;
   int mine = 0;
-  for (int j = j0; j < min(j0 + per, r); ++j) mine += p.ccount[c0 + j];
-  int base = block_exclusive_scan(mine, warp_sums, nullptr);
-  for (int j = j0; j < min(j0 + per, r); ++j) {
-    at[j] = base;
-    if (blockIdx.x == 0) p.cbase[c0 + j] = base;
-    base += p.ccount[c0 + j];
+  for (int g = g0; g < min(g0 + per, ng); ++g) mine += size(g);
+  int total = 0;
+  int base = block_exclusive_scan(mine, warp_sums, &total);
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.lsize[u] = total;
+  for (int g = g0; g < min(g0 + per, ng); ++g) {
+    at[g] = base;
+    if (blockIdx.x == 0) p.lbase[slot(g)] = base;
+    base += size(g);
   }
-  if (a >= r) {                        // only after a failed assignment
+  if (a >= r || o >= r) {                    // only after a failed assignment
     report_status(p.status, kStatusBadIndex);
-    a = -1;
+    a = o = -1;
   }
-  const int rank = a >= 0 ? atomicAdd(&cnt[a], 1) : 0;
+  if (!kMembers && a == o) a = o = -1;       // not moved
+  const int ra = a >= 0 ? atomicAdd(&cnt[a], 1) : 0;
+  const int ro = o >= 0 ? atomicAdd(&cnt[r + o], 1) : 0;
   __syncthreads();
-  for (int j = threadIdx.x; j < r; j += kScatterThreads)
-    if (cnt[j] > 0) at[j] += atomicAdd(p.cursor + c0 + j, cnt[j]);
+  for (int g = threadIdx.x; g < ng; g += kScatterThreads)
+    if (cnt[g] > 0) at[g] += atomicAdd(p.cursor + slot(g), cnt[g]);
   __syncthreads();
-  if (a < 0) return;
-  const int64_t off = int64_t(at[a]) + rank;
-  if (off < 0 || off >= p.s) {         // counts inconsistent with the assignment: the same
-    report_status(p.status, kStatusBadIndex);
-    return;
-  }
-  p.members[int64_t(u) * p.s + off] = int32_t(pos);
+  auto put = [&](int off) {
+    if (off < 0 || off >= 2 * p.s) {         // counts inconsistent with the assignment: the same
+      report_status(p.status, kStatusBadIndex);
+      return;
+    }
+    p.list[2 * int64_t(u) * p.s + off] = int32_t(pos);
+  };
+  if (a >= 0) put(at[a] + ra);
+  if (o >= 0) put(at[r + o] + ro);
 }
 
 // New centre = mean key of its members; on the last iteration also the mean
@@ -1128,24 +1145,12 @@ struct RowSum {
   __device__ __forceinline__ bool out_of_range() const { return (left & 0xff800000u) != 0u; }
 };
 
-// values = false: the key sums (every pass); values = true: the value sums
-// (the last pass), a launch of their own so each keeps 8 rows in flight per
-// warp at full occupancy.
-// delta = 0: every member of the current lists.  Once few tokens move, the
-// key sums are updated instead (integer sums: the update is exact):
-// delta = +1 adds the members of the current lists whose centre changed, and
-// delta = -1 subtracts the members of the previous lists whose centre changed
-// (a bit of the moved-token bitmap per member; rows of movers only).  An
-// inexact value that joins raises the centre's flag; flags are kept while the
-// sums are (a flagged centre is summed again in fp64 from its members).
-// the moved-token bitmap of the iteration: token t's bit in word t / 32
-__global__ void k_lloyd_moved(LloydArgs p, int64_t n_tok) {
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const bool mv = t < n_tok && p.assign[t] != p.assign_prev[t];
-  const unsigned b = __ballot_sync(0xffffffffu, mv);
-  if ((threadIdx.x & 31) == 0 && t < n_tok) p.moved[t >> 5] = b;
-}
-
+// values = false: the key sums, updated by the tokens that joined a centre and
+// those that left one (the list of k_lloyd_scatter<false>; integer sums, so the
+// update is exact; in the first iteration every member joins).  values = true: the
+// value sums of every member (the last iteration, k_lloyd_scatter<true>).  A value
+// without a fixed-point form that joins raises the centre's flag, which stays for
+// the run (a flagged centre is summed again in fp64 from its members).
 // What bounds it: instruction issue (about 40 warp instructions per 256-byte row,
 // 2.7 issued per cycle) and DRAM, at 58 % of its rate.  A warp's rows arrive by
 // cp.async in a ring of kAccDepth batches of 8 (2 KB each), so that 8 KB per
@@ -1157,132 +1162,119 @@ __global__ void k_lloyd_moved(LloydArgs p, int64_t n_tok) {
 constexpr int kAccDepth = 4;
 constexpr size_t kAccSmem = size_t(kThreads / 32) * kAccDepth * 8 * kAsgRowBytes;
 
-template <bool values, int delta>
+template <bool values>
 __global__ void __launch_bounds__(kThreads, 3) k_lloyd_accum(LloydArgs p) {
-  static_assert(delta == 0 || !values, "value sums are taken in full");
   extern __shared__ __align__(128) uint8_t acc_raw[];
-  __shared__ int2 rows_s[kThreads / 32][kAccRowsPerWarp];   // (slot, position) of the rows to add
-  const int ul = blockIdx.y;
-  const int r = p.r_unit[ul];
+  __shared__ int rows_s[kThreads / 32][kAccRowsPerWarp];   // positions of the rows to add
+  const int u = blockIdx.y;
+  const int r = p.r_unit[u];
   if (r <= 0) return;
-  const int32_t* cb = (delta < 0 ? p.cbase_prev : p.cbase) + int64_t(ul) * p.rmax;
-  const int32_t* cc = (delta < 0 ? p.ccount_prev : p.ccount) + int64_t(ul) * p.rmax;
+  const int64_t c0 = int64_t(u) * p.rmax;
+  // groups of the list: joined (or every member) by centre, then left by centre
+  const int ng = values || !p.assign_prev ? r : 2 * r;
+  auto slot = [&](int g) { return 2 * c0 + (g < r ? g : p.rmax + g - r); };
   // (the clamps below only act after a failed assignment, whose status is raised)
-  const int n_mem = min(cb[r - 1] + cc[r - 1], int(p.s));
+  const int n_list = int(min(int64_t(p.lsize[u]), 2 * p.s));
+  auto start = [&](int g) { return p.lbase[slot(g)]; };
+  auto end = [&](int g) { return g + 1 < ng ? start(g + 1) : n_list; };
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int lo = blockIdx.x * kAccRows + w * kAccRowsPerWarp;
-  if (lo >= n_mem) return;
-  const int hi = min(n_mem, lo + kAccRowsPerWarp);
-  const int32_t* mem = (delta < 0 ? p.members_prev : p.members) + int64_t(ul) * p.s;
-  const __nv_bfloat16* X = (values ? p.V : p.K) + int64_t(ul) * p.s * kHeadDim;
-  // the rows to add, in slot order: all, or those whose token moved.  A member
-  // position outside the unit only follows a failed assignment (its status is
-  // raised): row 0 is read instead of leaving the array
-  int2* rows = rows_s[w];
-  int n = 0;
-#pragma unroll
-  for (int k = 0; k < kAccRowsPerWarp / 32; ++k) {
-    const int i = lo + 32 * k + lane;
-    int pos = i < hi ? mem[i] : 0;
-    pos = uint32_t(pos) < uint32_t(p.s) ? pos : 0;
-    bool take = i < hi;
-    if constexpr (delta != 0) {
-      const int64_t t = int64_t(ul) * p.s + pos;
-      take = take && ((p.moved[t >> 5] >> (t & 31)) & 1u);
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, take);
-    if (take) rows[n + __popc(bal & ((1u << lane) - 1u))] = make_int2(i, pos);
-    n += __popc(bal);
-  }
-  if (n == 0) return;
-  __syncwarp();
-  const uint32_t ring = smem_u32(acc_raw) + uint32_t(w * kAccDepth * 8 * kAsgRowBytes);
-  const uint2* ringp = reinterpret_cast<const uint2*>(acc_raw + w * kAccDepth * 8 * kAsgRowBytes) + lane;
-  // rows 8b .. 8b + 7 into stage b % kAccDepth: half a warp per row
-  auto issue = [&](int b) {
-#pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-      const int x = 8 * b + q + (lane >> 4);
-      if (x < n)
-        cp_async16(ring + uint32_t(((b % kAccDepth) * 8 + q + (lane >> 4)) * kAsgRowBytes + (lane & 15) * 16),
-                   X + int64_t(rows[x].y) * kHeadDim + 8 * (lane & 15), 16u);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-#pragma unroll
-  for (int b = 0; b < kAccDepth; ++b) issue(b);
-  // the centre holding slot rows[0]: the last j with cbase[j] <= it (it is
-  // never empty: an empty centre shares its cbase with the next one)
-  int j = 0;
-  for (int step = 1 << (31 - __clz(max(r - 1, 1))); step > 0; step >>= 1)
-    if (j + step < r && cb[j + step] <= rows[0].x) j += step;
-  int bnd = cb[j] + cc[j];
-  const int64_t m0 = int64_t(ul) * p.rmax * 2 * kHeadDim + (values ? kHeadDim : 0) + lane;
-  unsigned long long* ms = reinterpret_cast<unsigned long long*>(p.msum) + m0;
-  unsigned long long* ts = reinterpret_cast<unsigned long long*>(p.tsum) + m0;
-  RowSum sum;
-  sum.reset();
-  int x0 = 0;                     // first of the rows in the sums
-  // the lane's sums into centre jj's totals (dim 4 lane + q at 32 q + lane, so
-  // that a warp's additions meet whole sectors)
-  auto flush = [&](int jj) {
-    unsigned long long* m = ms + int64_t(jj) * 2 * kHeadDim;
-    const long long v[4] = {sum_total(sum.a.s.x, sum.a.t.x), sum_total(sum.a.s.y, sum.a.t.y),
-                            sum_total(sum.b.s.x, sum.b.t.x), sum_total(sum.b.s.y, sum.b.t.y)};
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      atomicAdd(m + 32 * q, static_cast<unsigned long long>(delta < 0 ? -v[q] : v[q]));
-    const bool bad = __any_sync(0xffffffffu, sum.bad || sum.out_of_range());
-    if (sum.dropped) {
-      unsigned long long* t = ts + int64_t(jj) * 2 * kHeadDim;
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (sum.tail[q] != 0)
-          atomicAdd(t + 32 * q, static_cast<unsigned long long>(delta < 0 ? -sum.tail[q] : sum.tail[q]));
-    }
-    if ((sum.dropped || bad) && lane == 0)
-      atomicOr(p.mflag + int64_t(ul) * p.rmax + jj, (sum.dropped ? kSumTails : 0u) | (bad ? kSumFp64 : 0u));
-    sum.reset();
-  };
-  for (int b = 0; 8 * b < n; ++b) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kAccDepth - 1) : "memory");
+  const __nv_bfloat16* X = (values ? p.V : p.K) + int64_t(u % p.UL) * p.s * kHeadDim;
+  int* rows = rows_s[w];
+  for (int lo = blockIdx.x * kAccRows + w * kAccRowsPerWarp; lo < n_list; lo += gridDim.x * kAccRows) {
+    const int n = min(n_list - lo, kAccRowsPerWarp);
+    // (a position outside the unit only follows a failed assignment: row 0 is
+    // read instead of leaving the array)
     __syncwarp();
-    const uint2* st = ringp + (b % kAccDepth) * 8 * 32 - 8 * b * 32;      // row x at st + 32 x
-    const int xe = min(n, 8 * b + 8);
-    for (int x = 8 * b; x < xe;) {
-      const int i = delta == 0 ? lo + x : rows[x].x;
-      if (i >= bnd && j < r - 1) {                // warp-uniform: row x is of a later centre
-        if (x > x0) flush(j);
-        x0 = x;
-        do {
-          ++j;
-          bnd = cb[j] + cc[j];
-        } while (i >= bnd && j < r - 1);
+#pragma unroll
+    for (int k = 0; k < kAccRowsPerWarp / 32; ++k) {
+      const int x = 32 * k + lane;
+      const int pos = x < n ? p.list[2 * int64_t(u) * p.s + lo + x] : 0;
+      rows[x] = uint32_t(pos) < uint32_t(p.s) ? pos : 0;
+    }
+    __syncwarp();
+    const uint32_t ring = smem_u32(acc_raw) + uint32_t(w * kAccDepth * 8 * kAsgRowBytes);
+    const uint2* ringp = reinterpret_cast<const uint2*>(acc_raw + w * kAccDepth * 8 * kAsgRowBytes) + lane;
+    // rows 8b .. 8b + 7 into stage b % kAccDepth: half a warp per row
+    auto issue = [&](int b) {
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) {
+        const int x = 8 * b + q + (lane >> 4);
+        if (x < n)
+          cp_async16(ring + uint32_t(((b % kAccDepth) * 8 + q + (lane >> 4)) * kAsgRowBytes + (lane & 15) * 16),
+                     X + int64_t(rows[x]) * kHeadDim + 8 * (lane & 15), 16u);
       }
-      // rows of this centre: those before bnd (or the last centre's, all);
-      // movers' slots are not consecutive and are taken one by one
-      const int xs = delta != 0 ? x + 1 : (j < r - 1 ? min(xe, bnd - lo) : xe);
-      for (; x + 4 <= xs; x += 4) sum.add<4>(st + 32 * x);
-      for (; x < xs; ++x) sum.add<1>(st + 32 * x);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int b = 0; b < kAccDepth; ++b) issue(b);
+    // the group holding slot lo: the last one that starts at or before it (it is
+    // never empty: an empty group starts with the next one)
+    int j = 0;
+    for (int step = 1 << (31 - __clz(max(ng - 1, 1))); step > 0; step >>= 1)
+      if (j + step < ng && start(j + step) <= lo) j += step;
+    int bnd = end(j) - lo;          // the row after the group's last
+    const int64_t m0 = c0 * 2 * kHeadDim + (values ? kHeadDim : 0) + lane;
+    unsigned long long* ms = reinterpret_cast<unsigned long long*>(p.msum) + m0;
+    unsigned long long* ts = reinterpret_cast<unsigned long long*>(p.tsum) + m0;
+    RowSum sum;
+    sum.reset();
+    // the lane's sums into group jj's centre (dim 4 lane + q at 32 q + lane, so
+    // that a warp's additions meet whole sectors)
+    auto flush = [&](int jj) {
+      const bool left = jj >= r;
+      const int c = left ? jj - r : jj;
+      unsigned long long* m = ms + int64_t(c) * 2 * kHeadDim;
+      const long long v[4] = {sum_total(sum.a.s.x, sum.a.t.x), sum_total(sum.a.s.y, sum.a.t.y),
+                              sum_total(sum.b.s.x, sum.b.t.x), sum_total(sum.b.s.y, sum.b.t.y)};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) atomicAdd(m + 32 * q, static_cast<unsigned long long>(left ? -v[q] : v[q]));
+      const bool bad = __any_sync(0xffffffffu, sum.bad || sum.out_of_range());
+      if (sum.dropped) {
+        unsigned long long* t = ts + int64_t(c) * 2 * kHeadDim;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (sum.tail[q] != 0)
+            atomicAdd(t + 32 * q, static_cast<unsigned long long>(left ? -sum.tail[q] : sum.tail[q]));
+      }
+      if ((sum.dropped || bad) && lane == 0)
+        atomicOr(p.mflag + c0 + c, (sum.dropped ? kSumTails : 0u) | (bad ? kSumFp64 : 0u));
+      sum.reset();
+    };
+    for (int b = 0; 8 * b < n; ++b) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kAccDepth - 1) : "memory");
+      __syncwarp();
+      const uint2* st = ringp + (b % kAccDepth) * 8 * 32 - 8 * b * 32;      // row x at st + 32 x
+      const int xe = min(n, 8 * b + 8);
+      for (int x = 8 * b; x < xe;) {
+        if (x >= bnd && j < ng - 1) {               // warp-uniform: row x is of a later group
+          if (x > 0) flush(j);
+          do {
+            ++j;
+            bnd = end(j) - lo;
+          } while (x >= bnd && j < ng - 1);
+        }
+        const int xs = j < ng - 1 ? min(xe, bnd) : xe;
+        for (; x + 4 <= xs; x += 4) sum.add<4>(st + 32 * x);
+        for (; x < xs; ++x) sum.add<1>(st + 32 * x);
+      }
+      __syncwarp();
+      issue(b + kAccDepth);
     }
-    __syncwarp();
-    issue(b + kAccDepth);
+    flush(j);
   }
-  flush(j);
 }
 
 // One warp per centre, lane l on dims 4l..4l+3 (coalesced sums, centres and
 // entries); ||c||^2 of the fp32 centre by a butterfly (the certification
 // bounds its rounding for any summation order).
-// keep: the key sums and flags stay for the next pass's update (delta
-// accumulation); otherwise both halves of the sums and the flag are cleared.
-__global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, int final_pass, int keep) {
+__global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, int final_pass) {
   const int lane = threadIdx.x & 31;
-  const int j = blockIdx.x * kFinWarps + (threadIdx.x >> 5), ul = blockIdx.y;
-  const int r = p.r_unit[ul];
+  const int j = blockIdx.x * kFinWarps + (threadIdx.x >> 5), u = blockIdx.y, ul = u % p.UL;
+  const int r = p.r_unit[u];
   if (j >= r) return;
-  const int64_t uj = int64_t(ul) * p.rmax + j;
-  const int cnt = p.ccount[uj];
+  const int64_t uj = int64_t(u) * p.rmax + j;
+  const int32_t* mc = p.mcount + 2 * int64_t(u) * p.rmax + j;
+  const int cnt = (p.assign_prev ? p.ccount[uj] : 0) + mc[0] - mc[p.rmax];
   const uint32_t flag = p.mflag[uj];
   const bool exact = flag == 0u;
   // dim 4 lane + q of the key sums at 32 q, of the value sums at kHeadDim + 32 q
@@ -1326,7 +1318,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     // fp64 sums over the unit's tokens in order
 #pragma unroll
     for (int q = 0; q < 4; ++q) tk[q] = tv[q] = 0.0;
-    const int32_t* as = p.assign + int64_t(ul) * p.s;
+    const int32_t* as = p.assign + int64_t(u) * p.s;
     const __nv_bfloat16* Kd = p.K + int64_t(ul) * p.s * kHeadDim + 4 * lane;
     const __nv_bfloat16* Vd = p.V + int64_t(ul) * p.s * kHeadDim + 4 * lane;
     for (int64_t t0 = 0; t0 < p.s; t0 += 32) {
@@ -1355,7 +1347,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
       mv[q] = final_pass ? tv[q] / cd : 0.0;
     }
   }
-  if (!keep) {
+  if (final_pass) {                   // the next run starts from zero
 #pragma unroll
     for (int q = 0; q < 4; ++q) ms[32 * q] = ms[kHeadDim + 32 * q] = 0;
     if (!exact) {
@@ -1373,7 +1365,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
       c64[q] = mk[q];
       c32[q] = cf[q];
     }
-    split_planes(p, ul, j, lane, cf);
+    split_planes(p, u, j, lane, cf);
   } else {                            // an empty centre keeps its place
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -1385,7 +1377,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
   if (final_pass) {
-    const int64_t e = int64_t(ul) * p.ent_stride + p.ent_off + j;
+    const int64_t e = int64_t(ul) * p.ent_stride + p.run_off[u / p.UL] + j;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       p.kbar[e * kHeadDim + 4 * lane + q] = __double2bfloat16(mk[q]);
@@ -1393,10 +1385,11 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     }
     if (lane == 0) p.ecount[e] = cnt;
   }
-  __syncwarp();                       // every lane has read mflag
+  __syncwarp();                       // every lane has read mflag and ccount
   if (lane == 0) {
     p.cnorm[uj] = n;
-    if (!keep) p.mflag[uj] = 0u;
+    p.ccount[uj] = cnt;
+    if (final_pass) p.mflag[uj] = 0u;
   }
 }
 

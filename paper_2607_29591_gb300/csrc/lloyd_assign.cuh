@@ -50,9 +50,10 @@
 // warps work on different steps at once; 24 warps run with the registers moved
 // (setmaxnreg) to the column warps.
 //
-// Members are counted in ccount by global reductions; where a unit has at most
-// 64 centres, so that many tokens meet in one, each decider counts in shared
-// memory and adds to ccount when it leaves the unit.  Every wait is
+// Tokens that joined and left a centre are counted in mcount by global
+// reductions; where a unit has at most 64 centres, so that many tokens meet in
+// one, each decider counts in shared memory and adds when it leaves the unit.
+// Every wait is
 // bounded; a wait that gives up raises kStatusWaitTimeout and an abort flag that
 // ends every other wait.  No barrier is shared by warps that may leave.
 //
@@ -122,7 +123,7 @@ struct AsgShared {
   int xrk[2][kTile];                                   // and ranks
   float kn[kAsgInfo][kTile];                           // the tile's key norms and ranks
   int rk[kAsgInfo][kTile];
-  int cnt[4][kAsgCnt];                                 // the deciders' member counts
+  int cnt[4][2][kAsgCnt];                              // the deciders' counts: joined, left
   int tinfo[2][2];                                     // per TMEM buffer: max ||c||, norm buffer
   uint32_t abort;
   int amb_n;                                           // listed tokens
@@ -332,7 +333,7 @@ struct AsgCand {
 // against the centres [seg0, seg0 + segw) of each unit (segw <= 256, a multiple
 // of 16; units with fewer centres are skipped).  The launch that sees a unit's
 // last centre decides its tokens: assign (centre index, -1 for tokens outside
-// E), member counts (ccount), and the list of tokens left (amb: the CTA's
+// E), the counts of moves (mcount), and the list of tokens left (amb: the CTA's
 // entries from tile g0's place on, amb_count).  p.knorm holds the key norms.
 // NB: 16-column blocks per column warp, segw <= 64 NB.
 template <int NB>
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
   const int64_t n_all = int64_t(p.n_units) * p.ntiles;   // below 2^31 (the tokens are)
   const int g0 = int(n_all * blockIdx.x / gridDim.x), g1 = int(n_all * (blockIdx.x + 1) / gridDim.x);
 
-  for (int i = tid; i < 4 * kAsgCnt; i += kAsgThreads) sh.cnt[0][i] = 0;
+  for (int i = tid; i < 8 * kAsgCnt; i += kAsgThreads) sh.cnt[0][0][i] = 0;
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sh.full[i], 2);
@@ -492,10 +493,12 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
           }
         }
         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sh.key_full[slot])) : "memory");
-        if (seg0 > 0) {                                // the candidates so far into L2, a line a lane
-          const int64_t t0 = int64_t(cl.tile) * kTile + 16 * (lane & 7);
-          if (lane < 8 && t0 < p.s)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.cand + int64_t(cl.u) * p.s + t0));
+        // the candidates and the centres so far into L2, a line a lane
+        const int64_t t0 = int64_t(cl.tile) * kTile + (lane < 8 ? 16 * lane : 32 * (lane & 3));
+        if (t0 < p.s) {
+          if (lane < 8 && seg0 > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.cand + int64_t(cl.u) * p.s + t0));
+          if (lane >= 8 && lane < 12 && p.assign_prev)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.assign_prev + int64_t(cl.u) * p.s + t0));
         }
       }
       if (!ok && lane == 0) asg_raise(&sh.abort, p.status);
@@ -607,14 +610,14 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
       // ---------------- deciders ----------------
       const int q = warp - kAsgDecide, tok = 32 * q + lane;
       int t = 0, cur_u = -1, keep = 0;
-      // the warp's member counts of the unit so far into ccount
+      // the warp's counts of the unit so far into mcount
       auto flush = [&]() {
         __syncwarp();
         if (cur_u >= 0 && p.r_unit[cur_u] <= kAsgCnt)
-          for (int i = lane; i < kAsgCnt; i += 32) {
-            const int c = sh.cnt[q][i];
-            if (c != 0) atomicAdd(p.ccount + int64_t(cur_u) * p.rmax + i, c);
-            sh.cnt[q][i] = 0;
+          for (int i = lane; i < 2 * kAsgCnt; i += 32) {
+            const int h = i / kAsgCnt, j = i % kAsgCnt, c = sh.cnt[q][h][j];
+            if (c != 0) atomicAdd(p.mcount + (2 * int64_t(cur_u) + h) * p.rmax + j, c);
+            sh.cnt[q][h][j] = 0;
           }
         __syncwarp();
       };
@@ -627,6 +630,8 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
           cur_u = u;
           keep = int(unit_budget(p.budgets, u % p.UL, p.budget)) - r - p.recent;   // ranked tokens from here on are in E
         }
+        const int64_t tix = int64_t(u) * p.s + pos;
+        const int old = mine && p.assign_prev ? p.assign_prev[tix] : -1;   // (in L2 by now)
         ok = asg_wait(&sh.xch_full[b], uint32_t((t >> 1) & 1), &sh.abort);
         if (__any_sync(0xffffffffu, !ok)) break;
         const float ww = sh.xw[b][tok];
@@ -642,7 +647,6 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
         AsgCand cd = join(AsgCand::unpack(x0), AsgCand::unpack(x1));
         cd = join(cd, AsgCand::unpack(x2));
         cd = join(cd, AsgCand::unpack(x3));
-        const int64_t tix = int64_t(u) * p.s + pos;
         if (seg0 > 0 && mine) cd = join(AsgCand::unpack(p.cand[tix]), cd);   // the segments before
         if (r > seg0 + segw) {                              // more centres in the next launch
           if (mine) p.cand[tix] = cd.pack();
@@ -666,8 +670,16 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
           // decided, written and counted by k_lloyd_resolve
         } else if (ev) {
           p.assign[tix] = cd.first;
-          if (r <= kAsgCnt) atomicAdd(&sh.cnt[q][cd.first], 1);
-          else atomicAdd(p.ccount + int64_t(u) * p.rmax + cd.first, 1);
+          if (cd.first != old) {
+            const int64_t c0 = 2 * int64_t(u) * p.rmax;
+            if (r <= kAsgCnt) {
+              atomicAdd(&sh.cnt[q][0][cd.first], 1);
+              if (old >= 0) atomicAdd(&sh.cnt[q][1][min(old, kAsgCnt - 1)], 1);
+            } else {
+              atomicAdd(p.mcount + c0 + cd.first, 1);
+              if (old >= 0) atomicAdd(p.mcount + c0 + p.rmax + min(old, r - 1), 1);
+            }
+          }
         } else if (mine) {
           p.assign[tix] = -1;
         }
@@ -698,7 +710,7 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
 // for |c32 - c64| <= u ||c||; the rest is slack for using d32 in place of D).
 // The fp32 best decides unless another candidate's interval
 // [d32_j - b_j, d32_j + b_j] reaches the best's; those few are re-evaluated in
-// fp64, ties to the lower index.  Writes assign and counts the member.
+// fp64, ties to the lower index.  Writes assign and counts the move.
 constexpr int kResWarps = 8;
 constexpr int kResChunk = 256;                  // distances held at once
 constexpr int kResMaxCtas = 1024;               // assignment CTAs (one list each)
@@ -863,7 +875,11 @@ __global__ void __launch_bounds__(kResWarps * 32) k_lloyd_resolve(LloydArgs p, i
         res = 0;
       }
       p.assign[int64_t(u) * p.s + pos] = res;
-      atomicAdd(p.ccount + int64_t(u) * p.rmax + res, 1);
+      const int old = p.assign_prev ? p.assign_prev[int64_t(u) * p.s + pos] : -1;
+      if (res != old) {
+        atomicAdd(p.mcount + 2 * int64_t(u) * p.rmax + res, 1);
+        if (old >= 0) atomicAdd(p.mcount + (2 * int64_t(u) + 1) * p.rmax + min(old, r - 1), 1);
+      }
     }
     __syncwarp();                                       // dl / jl are reused by the next token
   }
