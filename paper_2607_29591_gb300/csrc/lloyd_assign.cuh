@@ -61,7 +61,8 @@
 // adds 16 exact products to the fp32 accumulator with an error of at most
 // 17 * 2^-22 times the largest partial magnitude (<= P) even if it truncates to
 // 24 bits; 16 chained steps (both planes) give 272 * 2^-22 P = 1088u P, the split
-// e adds 256u P: taken as 2048u P.
+// e adds 256u P, |c1| + |c2| exceeds |c| by 2^-8: 1350u P, taken as 1440u P.  (A
+// bound three times as wide cost k_lloyd_resolve 1.7 to 2.1 times its time.)
 //
 // What bounds it: issue and the latency of a tile's steps (about 2.3 instructions
 // per cycle; the tensor pipe is active 28 % of the time at r = 51 and 54 % at 204,
@@ -420,12 +421,13 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
       tc_fence_before();
       asg_arrive(&sh.tmem_empty[b]);                         // TMEM buffer, tile info and norms are free
       const float d0 = fminf(min3(a[0], a[1], a[2]), a[3]);
-      // A distance is off by at most ee + 4u |d|: ee = 2 x (dot product
-      // 2 gam_tc ||c|| ||k|| + norm sum 2 gam ||c||^2 + fp32 centre 4u ||k||
-      // ||c||), ||c|| <= max ||c|| over the unit.  So the nearest centre's
-      // computed distance is within 2 ee + 4u (|d0| + |d|) of d0.
-      const float uu = 5.9604645e-8f, gam = 130.0f * uu, gam_tc = 2048.0f * uu;
-      const float ee = 2.0f * cm * ((2.0f * gam_tc + 4.0f * uu) * kn + 2.0f * gam * cm);
+      // A computed distance is off by at most ee + 4u |d| from the exact distance
+      // to the fp64 centre: ee = 2 x dot product (gam_tc ||c|| ||k||, and 2u for
+      // the fp32 centre) + norm sum gam ||c||^2 (130u, and 2u for the fp32 centre),
+      // ||c|| <= max ||c|| over the unit.  So the nearest centre's computed
+      // distance is within 2 ee + 4u (|d0| + |d|) of d0.
+      const float uu = 5.9604645e-8f, gam = 140.0f * uu, gam_tc = 1440.0f * uu;
+      const float ee = cm * (2.0f * gam_tc * kn + gam * cm);
       const float ww = 2.01f * ee;
       const float thr = d0 + asg_window(ww, d0);
       const float2 nthr = make_float2(-thr, -thr);
