@@ -306,7 +306,17 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   const int ntiles = int(cdiv(s, kTile));
   const int n_fit_rows = cfg.score_mode == RESKV_SCORE_OBS_POOL ? G * cfg.n_fit : 0;
   const int n_val_rows = proxy ? G * cfg.n_val : 0;
-  const int nchunks = int(cdiv(s, int64_t(kTile) * kValChunkTiles));
+  // Chunks of the validation targets: at most 16 tiles per CTA, and as many CTAs
+  // as fill whole waves of one CTA per SM.
+  const int row_blocks = int(cdiv(std::max(n_val_rows, 1), kValRows));
+  int64_t nchunks = 1;
+  for (int64_t wave = 1;; ++wave) {
+    nchunks = std::max<int64_t>(1, wave * c->num_sms / (int64_t(UL) * row_blocks));
+    if (cdiv(ntiles, nchunks) <= 16) break;
+  }
+  const int chunk_tiles = int(cdiv(ntiles, nchunks));
+  nchunks = cdiv(ntiles, chunk_tiles);
+  const int nparts = int(nchunks) * val_shape(std::max(n_val_rows, 1) - (row_blocks - 1) * kValRows).splits;
   // entry storage: one slice per run with r > 0
   std::vector<int32_t> run_off(std::max(ncol, 2), 0);
   int64_t ent_stride = 0;
@@ -392,9 +402,9 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     if (US < size_t(kTile)) S.get(&kpad, kTile * kHeadDim);
   }
   if (proxy) {
-    S.get(&vpart, size_t(UL) * n_val_rows * nchunks * kValRec);
+    S.get(&vpart, size_t(UL) * n_val_rows * nparts * kValRec);
     S.get(&oS, size_t(UL) * n_val_rows * kHeadDim);
-    S.get(&rowerr, size_t(UL) * n_val_rows);
+    S.get(&rowerr, size_t(UL) * ncol * n_val_rows);
     S.get(&losses, size_t(UL) * ncol);
   }
   bool ok = S.commit();
@@ -460,8 +470,8 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       set_smem(k_lloyd_assign<4>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_accum<false>, kAccSmem) != cudaSuccess ||
       set_smem(k_lloyd_accum<true>, kAccSmem) != cudaSuccess ||
-      set_smem(k_val_loss, kValSmem) != cudaSuccess ||
-      set_smem(k_val_full, kValSmem) != cudaSuccess)
+      set_smem(k_val_loss, kValSmemLoss) != cudaSuccess ||
+      set_smem(k_val_full, kValSmemFull) != cudaSuccess)
     return cleanup_fail(fail(RESKV_ERR_CUDA, "setting kernel shared-memory limits"));
 
   const double one_minus_delta = 1.0 - double(cfg.delta);
@@ -643,39 +653,25 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     if (proxy) {
       // ---- validation targets, candidates, choice of r ----
       timing_ok &= timer.mark(kStValTargets);
-      ValArgs va{K, V, Q, s, G, cfg.n_obs, cfg.n_val, n_val_rows, nchunks, vpart, oS};
-      k_val_full<<<dim3(nchunks, unsigned(cdiv(n_val_rows, kRowBlk)), UL), kThreads, kValSmem, stream>>>(va);
+      ValArgs va{K, V, Q, s, G, cfg.n_obs, cfg.n_val, n_val_rows, chunk_tiles, int(nchunks), nparts, vpart, oS};
+      k_val_full<<<dim3(unsigned(nchunks), unsigned(row_blocks), UL), kThreads, kValSmemFull, stream>>>(va);
       k_val_combine<<<dim3(n_val_rows, UL), kHeadDim, 0, stream>>>(va);
       RESKV_LAUNCH_CHECK("validation targets");
-      for (int run = 0; run < ncol; ++run) {
-        const int32_t* r_unit = r_runs + size_t(run) * UL;
-        auto r_most = [&](int k) {       // the largest r of candidate k (0: no unit has it)
-          int r_hi = 0;
-          for (int i = 0; i < UL; ++i) r_hi = std::max(r_hi, hr[size_t(k) * UL + i]);
-          return r_hi;
-        };
-        if (run > 0 && (run - 1) % n_batch == 0) {
-          const int n_run = std::min(n_batch, ncol - run);
-          int r_hi = 0;
-          for (int k = run; k < run + n_run; ++k) r_hi = std::max(r_hi, r_most(k));
-          if (r_hi > 0 && (st = lloyd_run(r_unit, run, n_run, r_hi)) != RESKV_OK) return cleanup_fail(st);
-        }
-        if (run > 0 && r_most(run) == 0) {
-          k_loss_reduce<<<unsigned(cdiv(UL, 128)), 128, 0, stream>>>(rowerr, losses, 0, UL,
-                                                                    ncol, run, r_unit);
-          RESKV_LAUNCH_CHECK("validation loss");
-          continue;
-        }
-        timing_ok &= timer.mark(kStValLoss);
-        LossArgs lo{K, V, Q, s, G, cfg.n_obs, cfg.n_val, n_val_rows, P, n_top, b, top, r_unit,
-                    kbar, vbar, ecount, ent_stride, run_off[run], cfg.beta, cfg.gate_mode,
-                    cfg.tau, cfg.alpha, cfg.g_min, cfg.g_fixed, oS, rowerr, cfg.softmax_mode,
-                    bl_d};
-        k_val_loss<<<dim3(unsigned(cdiv(n_val_rows, kRowBlk)), UL), kThreads, kValSmem, stream>>>(lo);
-        k_loss_reduce<<<unsigned(cdiv(UL, 128)), 128, 0, stream>>>(rowerr, losses, n_val_rows, UL,
-                                                                  ncol, run, r_unit);
-        RESKV_LAUNCH_CHECK("validation loss");
+      for (int run = 1; run < ncol; run += n_batch) {
+        const int n_run = std::min(n_batch, ncol - run);
+        int r_hi = 0;                    // (0: no unit of the layer has these candidates)
+        for (int i = 0; i < UL * n_run; ++i) r_hi = std::max(r_hi, hr[size_t(run) * UL + i]);
+        if (r_hi > 0 && (st = lloyd_run(r_runs + size_t(run) * UL, run, n_run, r_hi)) != RESKV_OK)
+          return cleanup_fail(st);
       }
+      timing_ok &= timer.mark(kStValLoss);
+      LossArgs lo{K, V, Q, s, UL, G, cfg.n_obs, cfg.n_val, n_val_rows, P, n_top, b, top, r_runs,
+                  kbar, vbar, ecount, ent_stride, run_off_d, cfg.beta, cfg.gate_mode,
+                  cfg.tau, cfg.alpha, cfg.g_min, cfg.g_fixed, oS, rowerr, cfg.softmax_mode, bl_d};
+      k_val_loss<<<dim3(unsigned(row_blocks), UL, ncol), kThreads, kValSmemLoss, stream>>>(lo);
+      k_loss_reduce<<<unsigned(cdiv(int64_t(UL) * ncol, 8)), 256, 0, stream>>>(rowerr, losses, n_val_rows, UL,
+                                                                             ncol, r_runs);
+      RESKV_LAUNCH_CHECK("validation loss");
       k_choose<<<unsigned(cdiv(UL, 128)), 128, 0, stream>>>(losses, ncol, r_runs, UL,
                                                            one_minus_delta, r_final, chosen);
       RESKV_LAUNCH_CHECK("choosing r");

@@ -19,35 +19,11 @@ namespace build {
 namespace cg = cooperative_groups;
 
 constexpr int kTile = 128;          // tokens per tile
-constexpr int kRowBlk = 32;         // query rows per block
 constexpr int kThreads = 256;       // 8 warps
 
 // ---------------------------------------------------------------------------
 // Shared-memory tiles
 // ---------------------------------------------------------------------------
-
-// Keys of a 128-token tile, fp32, dim-major, with the float4 column swizzled
-// by (dim / 8) so that the transposing stores spread over banks.
-__device__ __forceinline__ int kt_index(int k, int tok) {
-  return k * kTile + ((((tok >> 2) ^ ((k >> 3) & 7)) << 2) | (tok & 3));
-}
-
-// Load rows [tok0, tok0 + 128) of a [s, d] bf16 matrix into Kt (zeros past s).
-__device__ __forceinline__ void load_kt(float* Kt, const __nv_bfloat16* K, int64_t s, int64_t tok0) {
-  for (int it = 0; it < 8; ++it) {
-    const int idx = it * kThreads + threadIdx.x;
-    const int tok = idx >> 4, dc = idx & 15;
-    uint4 w = make_uint4(0, 0, 0, 0);
-    if (tok0 + tok < s) w = __ldg(reinterpret_cast<const uint4*>(K + (tok0 + tok) * kHeadDim) + dc);
-    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = bf16x2_to_float2(ws[j]);
-      Kt[kt_index(8 * dc + 2 * j, tok)] = f.x;
-      Kt[kt_index(8 * dc + 2 * j + 1, tok)] = f.y;
-    }
-  }
-}
 
 constexpr int kAsgRowBytes = kHeadDim * 2;  // one bf16 row of 128 dims
 
@@ -77,50 +53,6 @@ __device__ __forceinline__ void stage_key_tile(uint32_t ks_s, const __nv_bfloat1
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Load 32 query rows (scaled) into Qt[k][row]; rows >= n_rows are zero.
-// row r of the block is global row rowbase + r, read from rowptr(r).
-template <typename RowPtr>
-__device__ __forceinline__ void load_qt(float* Qt, int n_rows, float scale, RowPtr rowptr) {
-  for (int it = 0; it < 2; ++it) {
-    const int idx = it * kThreads + threadIdx.x;
-    const int row = idx >> 4, dc = idx & 15;
-    uint4 w = make_uint4(0, 0, 0, 0);
-    if (row < n_rows) w = __ldg(reinterpret_cast<const uint4*>(rowptr(row)) + dc);
-    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float2 f = bf16x2_to_float2(ws[j]);
-      Qt[(8 * dc + 2 * j) * kRowBlk + row] = f.x * scale;
-      Qt[(8 * dc + 2 * j + 1) * kRowBlk + row] = f.y * scale;
-    }
-  }
-}
-
-// S[4 rows][4 tokens] for warp w (rows 4w..4w+3) and lane (tokens 4l..4l+3).
-__device__ __forceinline__ void tile_logits(const float* Qt, const float* Kt, float S[4][4]) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) S[i][j] = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < kHeadDim; ++k) {
-    const float4 q = *reinterpret_cast<const float4*>(Qt + k * kRowBlk + 4 * w);
-    const float4 kk = *reinterpret_cast<const float4*>(Kt + k * kTile + ((lane ^ ((k >> 3) & 7)) << 2));
-    const float qa[4] = {q.x, q.y, q.z, q.w};
-    const float ka[4] = {kk.x, kk.y, kk.z, kk.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) S[i][j] = fmaf(qa[i], ka[j], S[i][j]);
-  }
-}
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1397,35 +1329,63 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
 // Validation proxy (Sec. 5.5.1, Eqs. valloss, valproxy; Alg. 1)
 // ---------------------------------------------------------------------------
 
-constexpr int kValChunkTiles = 16;           // 2048 tokens per CTA
 constexpr int kValRec = kHeadDim + 4;        // m, l, 2 pad, acc[d]: acc 16-byte aligned
+constexpr int kValRows = 128;                // query rows per CTA, at most
 
-struct ValArgs {
-  const __nv_bfloat16* K;
-  const __nv_bfloat16* V;
-  const __nv_bfloat16* Qobs;   // [UL*G, n_obs, d]
-  int64_t s;
-  int32_t G, n_obs, n_val, n_rows;     // n_rows = G * n_val, row = g * n_val + t
-  int32_t nchunks;
-  float* part;                 // [UL, n_rows, nchunks, kValRec]  (m, l, pad, acc)
-  float* oS;                   // [UL, n_rows, d]
+// Attention of the validation queries over many tokens on the tensor cores
+// (mma.sync m16n8k16, as the scores), shared by the targets (k_val_full) and the
+// candidates' losses (k_val_loss).  A CTA of 8 warps walks tiles of 128 key and
+// value rows (bf16, 256-byte rows XOR-swizzled for ldmatrix), two in flight by
+// cp.async.  The warps split the query rows in groups of 16 and, where there are
+// fewer than 8 groups, each tile's tokens between `splits` warps of a group.  A
+// warp takes 32 tokens at a time: logits (exact bf16 products, fp32 sums), an
+// online softmax in registers, and P V with the fp32 weights split into three
+// bf16 planes (p = p1 + p2 + p3 exactly), so no weight loses a bit.  The sums of
+// 32 tokens are formed apart and added to the running ones in fp32: longer chains
+// of tensor-core additions, which do not round to nearest, had twice the error of
+// the fp32 FMAs this replaces against 64 bits; so formed it is the same (mean error
+// of L_0 over 6 shapes 3.8e-7 of it, before and now).
+//
+// What bounds it: the legacy tensor-core rate (four times the products of one
+// bf16 plane) and the softmax's issue between the MMAs.  P V used to take fp32
+// FMAs from shared memory, with half of the warps idle during the logits:
+// targets of 64 units x 32 rows x 32K tokens 645 -> 320 us, of 32 units x 128 rows
+// x 128K tokens 4822 -> 1769 us; five columns of losses (b = 1024, batch 8) 508 ->
+// 142 us a layer, in one launch.
+struct ValState {
+  float O[16][4];                // numerators of rows g, g + 8 at dims 8 nt + 2 t4 (+1)
+  float m[2], l[2];              // reference maxima, this lane's share of the sums
+
+  __device__ __forceinline__ void reset() {
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) O[nt][0] = O[nt][1] = O[nt][2] = O[nt][3] = 0.f;
+    m[0] = m[1] = -INFINITY;
+    l[0] = l[1] = 0.f;
+  }
 };
 
-__device__ __forceinline__ const __nv_bfloat16* val_row(const ValArgs& p, int ul, int row) {
-  const int g = row / p.n_val, t = row % p.n_val;
-  return p.Qobs + ((int64_t(ul) * p.G + g) * p.n_obs + (p.n_obs - p.n_val) + t) * kHeadDim;
+// D = A * B, m16n8k16, bf16 inputs, fp32 result
+__device__ __forceinline__ void mma16816_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// Shared memory of the validation kernels (k_val_full, k_val_loss): the key
-// tile (bf16, 256-byte rows with the 16-byte chunks XOR-swizzled for
-// ldmatrix), the value tile (bf16 rows), the logits of the CTA's 32 query rows
-// (fp32, rows padded to 136 floats: the fragment stores are conflict free)
-// and P^T (fp32, swizzled).  Under 113 KB: two CTAs per SM.
-constexpr int kValSRow = kTile + 8;
-constexpr size_t kValOffV = size_t(kTile) * kAsgRowBytes;
-constexpr size_t kValOffS = kValOffV + size_t(kTile) * kAsgRowBytes;
-constexpr size_t kValOffP = kValOffS + size_t(kRowBlk) * kValSRow * 4;
-constexpr size_t kValSmem = kValOffP + size_t(kTile) * kRowBlk * 4;
+// How a CTA's warps share its rows and a tile's tokens.
+struct ValShape {
+  int groups;                    // groups of 16 rows: 1, 2, 4 or 8
+  int splits;                    // warps per group: min(4, 8 / groups)
+};
+
+__host__ __device__ inline ValShape val_shape(int n_rows) {
+  const int g = (n_rows + 15) / 16;
+  ValShape v;
+  v.groups = g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : 8;
+  v.splits = v.groups >= 2 ? 8 / v.groups : 4;
+  return v;
+}
 
 // A fragments (m16n8k16) of 16 query rows: row g and g + 8 of lane g = lane / 4
 // from rowptr(i) (nullptr: a zero row), unscaled bf16
@@ -1443,163 +1403,239 @@ __device__ __forceinline__ void val_afrag(RowPtr rowptr, int lane, uint32_t (&A)
   }
 }
 
-// The scaled logits (log2 domain) of the CTA's 32 rows against the staged key
-// tile into St: warp w < 4 takes rows 16 (w / 2).. and tokens 64 (w % 2)..
-// (tensor cores: exact bf16 products, fp32 sums); the other warps wait.
-__device__ __forceinline__ void val_tile_logits(uint32_t ks_s, const uint32_t (&A)[8][4], float* St) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (w >= 4) return;
-  float S[8][4];
-  obs_half_logits(ks_s, w & 1, lane, A, S);
-  const int g = lane >> 2, t4 = lane & 3, r0 = 16 * (w >> 1) + g;
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
-    const int tk = 64 * (w & 1) + 8 * nt + 2 * t4;
-    *reinterpret_cast<float2*>(St + r0 * kValSRow + tk) = make_float2(S[nt][0], S[nt][1]);
-    *reinterpret_cast<float2*>(St + (r0 + 8) * kValSRow + tk) = make_float2(S[nt][2], S[nt][3]);
-  }
-}
-
-// this thread's logits: rows 4w..4w+3, tokens 4l..4l+3
-__device__ __forceinline__ void val_read_logits(const float* St, float (&S)[4][4]) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float4 v = *reinterpret_cast<const float4*>(St + (4 * w + i) * kValSRow + 4 * lane);
-    S[i][0] = v.x;
-    S[i][1] = v.y;
-    S[i][2] = v.z;
-    S[i][3] = v.w;
-  }
-}
-
-// 128 rows of 256 bytes into a bf16 tile (rows swizzled for ldmatrix or
-// plain) by cp.async, one 16-byte chunk per copy; rowptr(i) = nullptr: zeros
-// (the copy then reads nothing from `any`, a valid global address)
-template <bool swz, typename RowPtr>
+// 128 rows of 256 bytes into a swizzled bf16 tile by cp.async, one 16-byte chunk
+// per copy; rowptr(i) = nullptr: zeros (the copy then reads nothing from `any`, a
+// valid global address)
+template <typename RowPtr>
 __device__ __forceinline__ void val_stage_rows(uint32_t dst, RowPtr rowptr, const __nv_bfloat16* any) {
   for (int idx = threadIdx.x; idx < kTile * 16; idx += blockDim.x) {
     const int row = idx >> 4, ch = idx & 15;
     const __nv_bfloat16* src = rowptr(row);
-    cp_async16(dst + (swz ? asg_swz(row, ch) : uint32_t(row * kAsgRowBytes + ch * 16)),
-               src ? src + 8 * ch : any, src ? 16u : 0u);
+    cp_async16(dst + asg_swz(row, ch), src ? src + 8 * ch : any, src ? 16u : 0u);
   }
 }
 
-// acc[i][d] += P^T[tok][row 4w + i] * V[tok][dim 4l + d] over the tile
-__device__ __forceinline__ void val_pv(const float* Pt, const __nv_bfloat16* Vb, float (&acc)[4][4]) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll 4
-  for (int tok = 0; tok < kTile; ++tok) {
-    const float4 pp = *reinterpret_cast<const float4*>(Pt + tok * kRowBlk + ((w ^ ((tok >> 2) & 7)) << 2));
-    const uint2 vw = *reinterpret_cast<const uint2*>(Vb + tok * kHeadDim + 4 * lane);
-    const float2 v01 = bf16x2_to_float2(vw.x), v23 = bf16x2_to_float2(vw.y);
-    const float pa[4] = {pp.x, pp.y, pp.z, pp.w};
-    const float va[4] = {v01.x, v01.y, v23.x, v23.y};
+// Tokens tk .. tk + 31 of the staged tile (keys at ks_s, values at vs_s) into
+// st; bias (log2 units, -inf: no token) per token of the tile, or NULL.
+__device__ __forceinline__ void val_block(ValState& st, const uint32_t (&A)[8][4], uint32_t ks_s, uint32_t vs_s,
+                                          int tk, const float* bias) {
+  const int lane = threadIdx.x & 31, t4 = lane & 3, mi = lane >> 3;
+  float S[4][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+  for (int nt = 0; nt < 4; ++nt) S[nt][0] = S[nt][1] = S[nt][2] = S[nt][3] = 0.f;
 #pragma unroll
-      for (int d = 0; d < 4; ++d) acc[i][d] = fmaf(pa[i], va[d], acc[i][d]);
+  for (int np = 0; np < 2; ++np) {
+    const int trow = tk + 16 * np + (mi >> 1) * 8 + (lane & 7);
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      uint32_t b0, b1, b2, b3;
+      ldsm_x4(ks_s + asg_swz(trow, 2 * ks + (mi & 1)), b0, b1, b2, b3);
+      mma16816(S[2 * np], A[ks][0], A[ks][1], A[ks][2], A[ks][3], b0, b1);
+      mma16816(S[2 * np + 1], A[ks][0], A[ks][1], A[ks][2], A[ks][3], b2, b3);
+    }
   }
+  const float scale = kLog2e * rsqrtf(float(kHeadDim));
+  float mx[2] = {st.m[0], st.m[1]};
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    float2 bs = make_float2(0.f, 0.f);
+    if (bias) bs = *reinterpret_cast<const float2*>(bias + tk + 8 * nt + 2 * t4);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      S[nt][2 * a] = fmaf(S[nt][2 * a], scale, bs.x);
+      S[nt][2 * a + 1] = fmaf(S[nt][2 * a + 1], scale, bs.y);
+      mx[a] = fmaxf(mx[a], fmaxf(S[nt][2 * a], S[nt][2 * a + 1]));
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], 1));
+    mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], 2));
+  }
+  if (__any_sync(0xffffffffu, mx[0] > st.m[0] || mx[1] > st.m[1])) {
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      // (no token so far and none here: mx = -inf, nothing to scale)
+      const float sc = mx[a] == -INFINITY ? 1.0f : exp2f(st.m[a] - mx[a]);
+      st.m[a] = mx[a];
+      st.l[a] *= sc;
+#pragma unroll
+      for (int nt = 0; nt < 16; ++nt) {
+        st.O[nt][2 * a] *= sc;
+        st.O[nt][2 * a + 1] *= sc;
+      }
+    }
+  }
+  float ls[4][2];
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        S[nt][2 * a + c] = st.m[a] == -INFINITY ? 0.f : exp2f(S[nt][2 * a + c] - st.m[a]);
+      ls[nt][a] = S[nt][2 * a] + S[nt][2 * a + 1];
+    }
+#pragma unroll
+  for (int a = 0; a < 2; ++a) st.l[a] += (ls[0][a] + ls[1][a]) + (ls[2][a] + ls[3][a]);
+  // the weights' three planes: n-tiles 2j, 2j + 1 are the A fragment of tokens 16j ..
+  uint32_t P[2][3][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      float x = S[2 * j + (f >> 1)][2 * (f & 1)], y = S[2 * j + (f >> 1)][2 * (f & 1) + 1];
+#pragma unroll
+      for (int pl = 0; pl < 3; ++pl) {
+        P[j][pl][f] = pack_bf16(x, y);
+        const float2 h = unpack_bf16(P[j][pl][f]);
+        x -= h.x;
+        y -= h.y;
+      }
+    }
+  const int vrow = tk + (mi & 1) * 8 + (lane & 7);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    uint32_t v[2][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      ldsm_x4_t(vs_s + asg_swz(vrow + 16 * j, 2 * q + (mi >> 1)), v[j][0], v[j][1], v[j][2], v[j][3]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                // the smallest products first
+      float T[4];
+      mma16816_zero(T, P[0][2], v[0][2 * h], v[0][2 * h + 1]);
+      mma16816(T, P[1][2][0], P[1][2][1], P[1][2][2], P[1][2][3], v[1][2 * h], v[1][2 * h + 1]);
+#pragma unroll
+      for (int pl = 1; pl >= 0; --pl)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          mma16816(T, P[j][pl][0], P[j][pl][1], P[j][pl][2], P[j][pl][3], v[j][2 * h], v[j][2 * h + 1]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) st.O[2 * q + h][e] += T[e];
+    }
+  }
+}
+
+// The warp's part of a staged tile.
+__device__ __forceinline__ void val_tile(ValState& st, const uint32_t (&A)[8][4], uint32_t ks_s, uint32_t vs_s,
+                                         int split, int splits, const float* bias) {
+  const int n = kTile / splits;                  // this warp's tokens
+  for (int tk = split * n; tk < (split + 1) * n; tk += 32) val_block(st, A, ks_s, vs_s, tk, bias);
+}
+
+// The finished state as records (m, l, pad, pad, acc) of the warp's 16 rows;
+// rec(row) is row's record.
+template <typename Rec>
+__device__ __forceinline__ void val_store(ValState& st, Rec rec) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    float l = st.l[a];
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    float* r = rec(g + 8 * a);
+    if (!r) continue;
+    if (t4 == 0) *reinterpret_cast<float2*>(r) = make_float2(st.m[a], l);
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt)
+      *reinterpret_cast<float2*>(r + 4 + 8 * nt + 2 * t4) = make_float2(st.O[nt][2 * a], st.O[nt][2 * a + 1]);
+  }
+}
+
+// Dynamic shared memory: two stages of a key and a value tile, their biases, and
+// (k_val_loss) the records of the main branch.
+constexpr size_t kValStage = 2 * size_t(kTile) * kAsgRowBytes;
+constexpr size_t kValOffBias = 2 * kValStage;
+constexpr size_t kValOffRec = kValOffBias + 2 * kTile * 4;
+constexpr size_t kValSmemFull = kValOffRec;
+constexpr size_t kValSmemLoss = kValOffRec + size_t(kThreads / 32) * 16 * kValRec * 4;
+static_assert(size_t(kThreads / 32) * 16 * kValRec * 4 <= kValOffBias, "the residual records reuse the stages");
+
+struct ValArgs {
+  const __nv_bfloat16* K;
+  const __nv_bfloat16* V;
+  const __nv_bfloat16* Qobs;   // [UL*G, n_obs, d]
+  int64_t s;
+  int32_t G, n_obs, n_val, n_rows;     // n_rows = G * n_val, row = g * n_val + t
+  int32_t chunk_tiles;         // tiles per CTA
+  int32_t nchunks;
+  int32_t nparts;              // partial records per row: chunks x the last row block's splits
+  float* part;                 // [UL, n_rows, nparts, kValRec]  (m, l, pad, acc)
+  float* oS;                   // [UL, n_rows, d]
+};
+
+// Query row `row` of unit ul: the last n_val observation rows of its heads.
+template <typename Args>
+__device__ __forceinline__ const __nv_bfloat16* val_row(const Args& p, int ul, int row) {
+  const int g = row / p.n_val, t = row % p.n_val;
+  return p.Qobs + ((int64_t(ul) * p.G + g) * p.n_obs + (p.n_obs - p.n_val) + t) * kHeadDim;
 }
 
 // o_S(q) over all s tokens for the validation queries (Eq. attn), per chunk
-__global__ void __launch_bounds__(kThreads, 2) k_val_full(ValArgs p) {
+__global__ void __launch_bounds__(kThreads, 1) k_val_full(ValArgs p) {
   extern __shared__ __align__(1024) uint8_t vraw[];
-  const uint32_t ks_s = smem_u32(vraw), vb_s = ks_s + uint32_t(kValOffV);
-  const __nv_bfloat16* Vb = reinterpret_cast<const __nv_bfloat16*>(vraw + kValOffV);
-  float* St = reinterpret_cast<float*>(vraw + kValOffS);
-  float* Pt = reinterpret_cast<float*>(vraw + kValOffP);
-  const int chunk = blockIdx.x, rb = blockIdx.y * kRowBlk, ul = blockIdx.z;
+  const uint32_t st_s = smem_u32(vraw);
+  float* bias_s = reinterpret_cast<float*>(vraw + kValOffBias);
+  const int chunk = blockIdx.x, rb = blockIdx.y * kValRows, ul = blockIdx.z;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const ValShape sh = val_shape(min(kValRows, p.n_rows - rb));
+  const int grp = w / sh.splits, split = w % sh.splits;
+  const bool active = grp < sh.groups;
+  const int r16 = rb + 16 * grp;
   uint32_t A[8][4];
-  if (w < 4) {
-    const int r16 = rb + 16 * (w >> 1);
-    val_afrag([&](int i) { return r16 + i < p.n_rows ? val_row(p, ul, r16 + i) : nullptr; }, lane, A);
-  }
-  float m[4], l[4], acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    m[i] = -INFINITY;
-    l[i] = 0.f;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) acc[i][d] = 0.f;
-  }
+  val_afrag([&](int i) { return active && r16 + i < p.n_rows ? val_row(p, ul, r16 + i) : nullptr; }, lane, A);
   const __nv_bfloat16* Ku = p.K + int64_t(ul) * p.s * kHeadDim;
   const __nv_bfloat16* Vu = p.V + int64_t(ul) * p.s * kHeadDim;
-  for (int tt = 0; tt < kValChunkTiles; ++tt) {
-    const int64_t tok0 = (int64_t(chunk) * kValChunkTiles + tt) * kTile;
-    if (tok0 >= p.s) break;
-    __syncthreads();
-    auto krow = [&](int i) { return tok0 + i < p.s ? Ku + (tok0 + i) * kHeadDim : nullptr; };
-    auto vrow = [&](int i) { return tok0 + i < p.s ? Vu + (tok0 + i) * kHeadDim : nullptr; };
-    val_stage_rows<true>(ks_s, krow, Ku);
-    val_stage_rows<false>(vb_s, vrow, Vu);
+  const int64_t tile0 = int64_t(chunk) * p.chunk_tiles;
+  const int n = int(min(int64_t(p.chunk_tiles), (p.s + kTile - 1) / kTile - tile0));
+  auto issue = [&](int t) {                      // tile t of the chunk into stage t & 1
+    if (t < n) {
+      const int64_t tok0 = (tile0 + t) * kTile;
+      const uint32_t dst = st_s + uint32_t((t & 1) * kValStage);
+      val_stage_rows(dst, [&](int i) { return tok0 + i < p.s ? Ku + (tok0 + i) * kHeadDim : nullptr; }, Ku);
+      val_stage_rows(dst + kTile * kAsgRowBytes,
+                     [&](int i) { return tok0 + i < p.s ? Vu + (tok0 + i) * kHeadDim : nullptr; }, Vu);
+      if (tok0 + kTile > p.s && threadIdx.x < kTile)
+        bias_s[(t & 1) * kTile + threadIdx.x] = tok0 + threadIdx.x < p.s ? 0.f : -INFINITY;
+    }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  };
+  ValState st;
+  st.reset();
+  issue(0);
+  for (int t = 0; t < n; ++t) {
+    issue(t + 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
-    val_tile_logits(ks_s, A, St);
+    const uint32_t ks_s = st_s + uint32_t((t & 1) * kValStage);
+    const bool ragged = (tile0 + t + 1) * kTile > p.s;
+    if (active)
+      val_tile(st, A, ks_s, ks_s + kTile * kAsgRowBytes, split, sh.splits,
+               ragged ? bias_s + (t & 1) * kTile : nullptr);
     __syncthreads();
-    float S[4][4];
-    val_read_logits(St, S);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float tmax = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (tok0 + 4 * lane + j >= p.s) S[i][j] = -INFINITY;
-        tmax = fmaxf(tmax, S[i][j]);
-      }
-      tmax = warp_max(tmax);
-      const float mn = fmaxf(m[i], tmax);
-      const float sc = exp2f(m[i] - mn);
-      l[i] *= sc;
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc[i][d] *= sc;
-      m[i] = mn;
-      float ps = 0.f;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        S[i][j] = exp2f(S[i][j] - mn);
-        ps += S[i][j];
-      }
-      l[i] += warp_sum(ps);
-    }
-    // P^T into shared memory: Pt[tok][rows], float4 column swizzled by (tok / 4)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int tok = 4 * lane + j;
-      *reinterpret_cast<float4*>(Pt + tok * kRowBlk + ((w ^ (lane & 7)) << 2)) =
-          make_float4(S[0][j], S[1][j], S[2][j], S[3][j]);
-    }
-    __syncthreads();
-    val_pv(Pt, Vb, acc);
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int row = rb + 4 * w + i;
-    if (row >= p.n_rows) continue;
-    float* out = p.part + ((int64_t(ul) * p.n_rows + row) * p.nchunks + chunk) * kValRec;
-    if (lane == 0) {
-      out[0] = m[i];
-      out[1] = l[i];
-    }
-    *reinterpret_cast<float4*>(out + 4 + 4 * lane) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-  }
+  if (active)
+    val_store(st, [&](int i) -> float* {
+      const int row = r16 + i;
+      return row < p.n_rows ? p.part + ((int64_t(ul) * p.n_rows + row) * p.nparts + chunk * sh.splits + split) * kValRec
+                            : nullptr;
+    });
 }
 
 __global__ void k_val_combine(ValArgs p) {
   const int row = blockIdx.x, ul = blockIdx.y, d = threadIdx.x;
-  const float* base = p.part + (int64_t(ul) * p.n_rows + row) * p.nchunks * kValRec;
+  const float* base = p.part + (int64_t(ul) * p.n_rows + row) * p.nparts * kValRec;
+  const int n = p.nchunks * val_shape(min(kValRows, p.n_rows - row / kValRows * kValRows)).splits;
   float m = -INFINITY, l = 0.f, a = 0.f;
-  for (int c = 0; c < p.nchunks; ++c) {
+#pragma unroll 4
+  for (int c = 0; c < n; ++c) {
     const float* q = base + int64_t(c) * kValRec;
-    const float cm = q[0], cl = q[1];
+    const float cm = q[0], cl = q[1], ca = q[4 + d];
     if (cl <= 0.f) continue;
     const float mn = fmaxf(m, cm);
     const float s0 = exp2f(m - mn), s1 = exp2f(cm - mn);
     l = l * s0 + cl * s1;
-    a = a * s0 + q[4 + d] * s1;
+    a = a * s0 + ca * s1;
     m = mn;
   }
   p.oS[(int64_t(ul) * p.n_rows + row) * kHeadDim + d] = a / l;
@@ -1610,191 +1646,166 @@ struct LossArgs {
   const __nv_bfloat16* V;
   const __nv_bfloat16* Qobs;
   int64_t s;
+  int32_t UL;
   int32_t G, n_obs, n_val, n_rows;
   int32_t recent, n_top, budget;
   const int32_t* top;          // [UL, n_top]
-  const int32_t* r_unit;       // [UL]
-  const __nv_bfloat16* kbar;   // [UL, ent_stride, d]
+  const int32_t* r_runs;       // [runs, UL]: r of every candidate; run 0: the pure main cache
+  const __nv_bfloat16* kbar;   // [UL, ent_stride, d], run k's entries at run_off[k]
   const __nv_bfloat16* vbar;
   const int32_t* ecount;
   int64_t ent_stride;
-  int32_t ent_off;
+  const int32_t* run_off;
   float beta;
   int32_t gate_mode;
   float tau, alpha, g_min, g_fixed;
   const float* oS;             // [UL, n_rows, d]
-  double* rowerr;              // [UL, n_rows]
+  double* rowerr;              // [runs, UL, n_rows]
   int32_t softmax_mode;        // decode rule of the losses (RESKV_SOFTMAX_*)
   const int32_t* budgets;      // [UL] per-unit budgets, or NULL (budget)
 };
 
-// ||o^(r)(q) - o_S(q)||^2 per validation query, with the decode rule of
-// Sec. 5.4 and the gate.  Tiled like k_val_full: a CTA takes 32 query rows of
-// a unit and walks the candidate's main slots (the kept ranked tokens, then
-// the recent window), then its residual entries (logit + beta ln c), each
-// gathered into shared memory once for all 32 rows (logits on the tensor
-// cores), with one online-softmax state per branch.  Dynamic shared memory:
-// kValSmem.
-struct LossState {
-  float m[4], l[4], acc[4][4];
-};
-
-// One 128-token tile (logits in St, V in Vb) into state st: logits + bias[j]
-// for this lane's tokens 4l + j (-inf: no token)
-__device__ __forceinline__ void loss_tile(const float* St, float* Pt, const __nv_bfloat16* Vb,
-                                          const float (&bias)[4], LossState& st) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float S[4][4];
-  val_read_logits(St, S);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float tmax = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      S[i][j] += bias[j];
-      tmax = fmaxf(tmax, S[i][j]);
-    }
-    tmax = warp_max(tmax);
-    const float mn = fmaxf(st.m[i], tmax);
-    // a tile with no token leaves the state as it is (mn = -inf)
-    const float sc = mn == -INFINITY ? 1.0f : exp2f(st.m[i] - mn);
-    st.l[i] *= sc;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) st.acc[i][d] *= sc;
-    st.m[i] = mn;
-    float ps = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      S[i][j] = mn == -INFINITY ? 0.f : exp2f(S[i][j] - mn);
-      ps += S[i][j];
-    }
-    st.l[i] += warp_sum(ps);
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int tok = 4 * lane + j;
-    *reinterpret_cast<float4*>(Pt + tok * kRowBlk + ((w ^ (lane & 7)) << 2)) =
-        make_float4(S[0][j], S[1][j], S[2][j], S[3][j]);
-  }
-  __syncthreads();
-  val_pv(Pt, Vb, st.acc);
-}
-
+// ||o^(r)(q) - o_S(q)||^2 per validation query and candidate, with the decode
+// rule of Sec. 5.4 and the gate.  A CTA takes up to 128 query rows of a unit and
+// one candidate: it walks the candidate's main slots (the kept ranked tokens,
+// then the recent window), then its residual entries (logit + beta ln c), each
+// gathered into shared memory once for all rows; one softmax state per branch,
+// the main one kept in shared memory while the residual one runs.
 __global__ void __launch_bounds__(kThreads, 1) k_val_loss(LossArgs p) {
   extern __shared__ __align__(1024) uint8_t vraw[];
-  const uint32_t ks_s = smem_u32(vraw), vb_s = ks_s + uint32_t(kValOffV);
-  const __nv_bfloat16* Vb = reinterpret_cast<const __nv_bfloat16*>(vraw + kValOffV);
-  float* St = reinterpret_cast<float*>(vraw + kValOffS);
-  float* Pt = reinterpret_cast<float*>(vraw + kValOffP);
-  const int rb = blockIdx.x * kRowBlk, ul = blockIdx.y;
+  const uint32_t st_s = smem_u32(vraw);
+  float* bias_s = reinterpret_cast<float*>(vraw + kValOffBias);
+  float* rec_m = reinterpret_cast<float*>(vraw + kValOffRec);     // [8 warps][16 rows][kValRec]
+  float* rec_r = reinterpret_cast<float*>(vraw);                  // the same, over the stages
+  const int rb = blockIdx.x * kValRows, ul = blockIdx.y, run = blockIdx.z;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = p.r_unit[ul];
+  const int r = p.r_runs[int64_t(run) * p.UL + ul];
+  if (run > 0 && r == 0) return;                 // the unit has no such candidate
   const int64_t bu = unit_budget(p.budgets, ul, p.budget);
   const int64_t m = r == 0 ? (bu < p.s ? bu : p.s) : bu - r;
   const int64_t keep = m - p.recent;
+  const ValShape sh = val_shape(min(kValRows, p.n_rows - rb));
+  const int grp = w / sh.splits, split = w % sh.splits;
+  const bool active = grp < sh.groups;
+  const int r16 = rb + 16 * grp;
   uint32_t A[8][4];
-  if (w < 4) {
-    const int r16 = rb + 16 * (w >> 1);
-    val_afrag([&](int i) -> const __nv_bfloat16* {
-      const int row = r16 + i;
-      if (row >= p.n_rows) return nullptr;
-      const int g = row / p.n_val, t = row % p.n_val;
-      return p.Qobs + ((int64_t(ul) * p.G + g) * p.n_obs + (p.n_obs - p.n_val) + t) * kHeadDim;
-    }, lane, A);
-  }
-  LossState sM, sR;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    sM.m[i] = sR.m[i] = -INFINITY;
-    sM.l[i] = sR.l[i] = 0.f;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) sM.acc[i][d] = sR.acc[i][d] = 0.f;
-  }
+  val_afrag([&](int i) { return active && r16 + i < p.n_rows ? val_row(p, ul, r16 + i) : nullptr; }, lane, A);
   const __nv_bfloat16* Ku = p.K + int64_t(ul) * p.s * kHeadDim;
   const __nv_bfloat16* Vu = p.V + int64_t(ul) * p.s * kHeadDim;
   const int32_t* top = p.top + int64_t(ul) * p.n_top;
-  // main slots: the ranked tokens kept, then the recent window
-  for (int64_t j0 = 0; j0 < m; j0 += kTile) {
-    auto pos = [&](int tok) -> int64_t {
-      const int64_t j = j0 + tok;
-      return j >= m ? -1 : (j < keep ? top[j] : (p.s - p.recent) + (j - keep));
-    };
-    __syncthreads();
-    val_stage_rows<true>(ks_s, [&](int tok) {
-      const int64_t q = pos(tok);
-      return q < 0 ? static_cast<const __nv_bfloat16*>(nullptr) : Ku + q * kHeadDim;
-    }, Ku);
-    val_stage_rows<false>(vb_s, [&](int tok) {
-      const int64_t q = pos(tok);
-      return q < 0 ? static_cast<const __nv_bfloat16*>(nullptr) : Vu + q * kHeadDim;
-    }, Vu);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    val_tile_logits(ks_s, A, St);
-    __syncthreads();
-    float bias[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) bias[j] = j0 + 4 * lane + j < m ? 0.f : -INFINITY;
-    loss_tile(St, Pt, Vb, bias, sM);
-  }
-  // residual entries: logit + beta ln c (log2 units); an empty entry is inert
-  const int64_t e0 = int64_t(ul) * p.ent_stride + p.ent_off;
-  for (int j0 = 0; j0 < r; j0 += kTile) {
-    __syncthreads();
-    val_stage_rows<true>(ks_s, [&](int tok) {
-      return j0 + tok < r ? p.kbar + (e0 + j0 + tok) * kHeadDim : static_cast<const __nv_bfloat16*>(nullptr);
-    }, Ku);
-    val_stage_rows<false>(vb_s, [&](int tok) {
-      return j0 + tok < r ? p.vbar + (e0 + j0 + tok) * kHeadDim : static_cast<const __nv_bfloat16*>(nullptr);
-    }, Vu);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    val_tile_logits(ks_s, A, St);
-    __syncthreads();
-    float bias[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int e = j0 + 4 * lane + j;
-      const int c = e < r ? p.ecount[e0 + e] : 0;
-      bias[j] = c > 0 ? p.beta * logf(float(c)) * kLog2e : -INFINITY;
-    }
-    loss_tile(St, Pt, Vb, bias, sR);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int row = rb + 4 * w + i;
-    float g_val = p.g_fixed;
-    if (p.gate_mode == RESKV_GATE_DYNAMIC) {
-      const float pmax = 1.0f / sM.l[i];
-      g_val = fmaxf(p.g_min, 1.0f / (1.0f + expf(-p.alpha * (p.tau - pmax))));
-    }
-    const float2 coef = branch_coefs(p.softmax_mode, g_val, sM.m[i], sM.l[i], sR.m[i], sR.l[i]);
-    float e = 0.f;
-    if (row < p.n_rows) {
-      const float* os = p.oS + (int64_t(ul) * p.n_rows + row) * kHeadDim + 4 * lane;
-#pragma unroll
-      for (int d = 0; d < 4; ++d) {
-        const float o = coef.x * sM.acc[i][d] + coef.y * sR.acc[i][d];
-        const float df = o - os[d];
-        e += df * df;
+  const int64_t e0 = int64_t(ul) * p.ent_stride + p.run_off[run];
+  const int n_main = int((m + kTile - 1) / kTile), n = n_main + (r + kTile - 1) / kTile;
+  auto issue = [&](int t) {                      // tile t into stage t & 1
+    if (t < n) {
+      const uint32_t dst = st_s + uint32_t((t & 1) * kValStage);
+      float* bias = bias_s + (t & 1) * kTile;
+      if (t < n_main) {
+        const int64_t j0 = int64_t(t) * kTile;
+        auto pos = [&](int i) -> int64_t {
+          const int64_t j = j0 + i;
+          return j >= m ? -1 : (j < keep ? top[j] : (p.s - p.recent) + (j - keep));
+        };
+        for (int idx = threadIdx.x; idx < kTile * 16; idx += kThreads) {
+          const int row = idx >> 4, ch = idx & 15;
+          const int64_t q = pos(row);
+          const int64_t at = q < 0 ? 0 : q * kHeadDim + 8 * ch;
+          cp_async16(dst + asg_swz(row, ch), Ku + at, q < 0 ? 0u : 16u);
+          cp_async16(dst + kTile * kAsgRowBytes + asg_swz(row, ch), Vu + at, q < 0 ? 0u : 16u);
+        }
+        if (threadIdx.x < kTile) bias[threadIdx.x] = j0 + threadIdx.x < m ? 0.f : -INFINITY;
+      } else {
+        const int j0 = (t - n_main) * kTile;
+        val_stage_rows(dst, [&](int i) { return j0 + i < r ? p.kbar + (e0 + j0 + i) * kHeadDim : nullptr; }, Ku);
+        val_stage_rows(dst + kTile * kAsgRowBytes,
+                       [&](int i) { return j0 + i < r ? p.vbar + (e0 + j0 + i) * kHeadDim : nullptr; }, Vu);
+        if (threadIdx.x < kTile) {
+          const int e = j0 + threadIdx.x;
+          const int c = e < r ? p.ecount[e0 + e] : 0;       // an empty entry is inert
+          bias[threadIdx.x] = c > 0 ? p.beta * logf(float(c)) * kLog2e : -INFINITY;
+        }
       }
     }
-    e = warp_sum(e);
-    if (lane == 0 && row < p.n_rows) p.rowerr[int64_t(ul) * p.n_rows + row] = double(e);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float* my_rec = rec_m + w * 16 * kValRec;
+  ValState st;
+  st.reset();
+  issue(0);
+  for (int t = 0; t < n; ++t) {
+    issue(t + 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    if (t == n_main && active) {                 // the residual branch begins
+      val_store(st, [&](int i) { return my_rec + i * kValRec; });
+      st.reset();
+    }
+    const uint32_t ks_s = st_s + uint32_t((t & 1) * kValStage);
+    if (active) val_tile(st, A, ks_s, ks_s + kTile * kAsgRowBytes, split, sh.splits, bias_s + (t & 1) * kTile);
+    __syncthreads();
+  }
+  if (active) {
+    if (n == n_main) {                           // no residual entries
+      val_store(st, [&](int i) { return my_rec + i * kValRec; });
+      st.reset();
+    }
+    val_store(st, [&](int i) { return rec_r + (w * 16 + i) * kValRec; });
+  }
+  __syncthreads();
+  // a warp per row: merge the splits of both branches, gate, error
+  for (int i = w; i < 16 * sh.groups; i += kThreads / 32) {
+    const int row = rb + i;
+    if (row >= p.n_rows) break;
+    float M[2], L[2];
+    float4 acc[2];
+#pragma unroll
+    for (int br = 0; br < 2; ++br) {
+      const float* rec = (br == 0 ? rec_m : rec_r) + ((i >> 4) * sh.splits * 16 + (i & 15)) * kValRec;
+      float mx = -INFINITY, l = 0.f;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < sh.splits; ++k) mx = fmaxf(mx, rec[k * 16 * kValRec]);
+      for (int k = 0; k < sh.splits; ++k) {
+        const float* q = rec + k * 16 * kValRec;
+        if (!(q[1] > 0.f)) continue;
+        const float sc = exp2f(q[0] - mx);
+        const float4 v = *reinterpret_cast<const float4*>(q + 4 + 4 * lane);
+        l += q[1] * sc;
+        a.x += v.x * sc;
+        a.y += v.y * sc;
+        a.z += v.z * sc;
+        a.w += v.w * sc;
+      }
+      M[br] = mx;
+      L[br] = l;
+      acc[br] = a;
+    }
+    float g_val = p.g_fixed;
+    if (p.gate_mode == RESKV_GATE_DYNAMIC) {
+      const float pmax = 1.0f / L[0];            // M[0] is the largest main logit
+      g_val = fmaxf(p.g_min, 1.0f / (1.0f + expf(-p.alpha * (p.tau - pmax))));
+    }
+    const float2 coef = branch_coefs(p.softmax_mode, g_val, M[0], L[0], M[1], L[1]);
+    const float4 os = *reinterpret_cast<const float4*>(p.oS + (int64_t(ul) * p.n_rows + row) * kHeadDim + 4 * lane);
+    const float dx = coef.x * acc[0].x + coef.y * acc[1].x - os.x, dy = coef.x * acc[0].y + coef.y * acc[1].y - os.y;
+    const float dz = coef.x * acc[0].z + coef.y * acc[1].z - os.z, dw = coef.x * acc[0].w + coef.y * acc[1].w - os.w;
+    const float e = warp_sum(dx * dx + dy * dy + dz * dz + dw * dw);
+    if (lane == 0) p.rowerr[(int64_t(run) * p.UL + ul) * p.n_rows + row] = double(e);
   }
 }
 
-// L_r = mean of the per-query errors (rows in order, fp64); +inf for a unit
-// without a candidate in this column (r_unit = 0 in a column c > 0)
+// L_r = mean of the per-query errors (fp64; a warp per unit and candidate); +inf
+// for a unit without a candidate in this column (r = 0 in a column c > 0)
 __global__ void k_loss_reduce(const double* rowerr, double* losses, int n_rows, int UL, int ncol,
-                              int col, const int32_t* r_unit) {
-  const int ul = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ul >= UL) return;
+                              const int32_t* r_runs) {
+  const int i = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (i >= UL * ncol) return;
+  const int col = i / UL, ul = i % UL;
+  const bool none = col > 0 && r_runs[i] == 0;
   double acc = 0.0;
-  for (int i = 0; i < n_rows; ++i) acc += rowerr[int64_t(ul) * n_rows + i];
-  losses[int64_t(ul) * ncol + col] = (col > 0 && r_unit[ul] == 0) ? INFINITY : acc / double(n_rows);
+  if (!none)
+    for (int k = lane; k < n_rows; k += 32) acc += rowerr[int64_t(i) * n_rows + k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) losses[int64_t(ul) * ncol + col] = none ? INFINITY : acc / double(n_rows);
 }
 
 // r* = argmin_{r>0} L_r (ties -> smaller r: columns hold ascending r); keep it
