@@ -468,8 +468,10 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       set_smem(k_lloyd_assign<2>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<3>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<4>, kAsgSmemMax) != cudaSuccess ||
-      set_smem(k_lloyd_accum<false>, kAccSmem) != cudaSuccess ||
-      set_smem(k_lloyd_accum<true>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false, true>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<true, true>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<false, false>, kAccSmem) != cudaSuccess ||
+      set_smem(k_lloyd_accum<true, false>, kAccSmem) != cudaSuccess ||
       set_smem(k_val_loss, kValSmemLoss) != cudaSuccess ||
       set_smem(k_val_full, kValSmemFull) != cudaSuccess)
     return cleanup_fail(fail(RESKV_ERR_CUDA, "setting kernel shared-memory limits"));
@@ -607,6 +609,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       la.n_units = U;
       la.run_off = run_off_d + run0;
       timing_ok &= timer.mark(kStLloyd);
+      const bool k16 = (reinterpret_cast<uintptr_t>(K) & 15u) == 0, v16 = (reinterpret_cast<uintptr_t>(V) & 15u) == 0;
       const unsigned gr = unsigned(cdiv((r_hi + 15) & ~15, kFinWarps));
       const unsigned asg_grid = unsigned(std::min<int64_t>(std::min(c->num_sms, kResMaxCtas), int64_t(U) * ntiles));
       // segments of at most 256 centres, of equal width
@@ -635,14 +638,14 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         }
         k_lloyd_resolve<<<unsigned(4 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
         k_lloyd_scatter<false><<<gs, kScatterThreads, size_t(r_hi) * 4 * sizeof(int), stream>>>(la);
-        k_lloyd_accum<false><<<ga, kThreads, kAccSmem, stream>>>(la);
+        (k16 ? k_lloyd_accum<false, true> : k_lloyd_accum<false, false>)<<<ga, kThreads, kAccSmem, stream>>>(la);
         if (last) {                       // the values of every member
           if (it > 0) {
             if (!clear(la.cursor, UR * rstride * 2))
               return fail(RESKV_ERR_CUDA, "clearing the list cursors");
             k_lloyd_scatter<true><<<gs, kScatterThreads, size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
           }
-          k_lloyd_accum<true><<<ga, kThreads, kAccSmem, stream>>>(la);
+          (v16 ? k_lloyd_accum<true, true> : k_lloyd_accum<true, false>)<<<ga, kThreads, kAccSmem, stream>>>(la);
         }
         k_lloyd_finish<<<dim3(unsigned(cdiv(r_hi, kFinWarps)), U), kFinWarps * 32, 0, stream>>>(la, last);
       }

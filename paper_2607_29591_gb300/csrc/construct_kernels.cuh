@@ -40,6 +40,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
                : "memory");
 }
 
+// the same for 8 bytes on an 8-byte boundary
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
 // Stage the bf16 keys of tokens tok0..tok0+127 as a swizzled [128][256 B]
 // tile (zeros past s); the copies complete at the caller's wait.
 __device__ __forceinline__ void stage_key_tile(uint32_t ks_s, const __nv_bfloat16* Ku, int64_t s,
@@ -1080,7 +1085,8 @@ struct RowSum {
 // values = false: the key sums, updated by the tokens that joined a centre and
 // those that left one (the list of k_lloyd_scatter<false>; integer sums, so the
 // update is exact; in the first iteration every member joins).  values = true: the
-// value sums of every member (the last iteration, k_lloyd_scatter<true>).  A value
+// value sums of every member (the last iteration, k_lloyd_scatter<true>).  wide: the
+// rows lie on a 16-byte boundary.  A value
 // without a fixed-point form that joins raises the centre's flag, which stays for
 // the run (a flagged centre is summed again in fp64 from its members).
 // What bounds it: instruction issue (about 40 warp instructions per 256-byte row,
@@ -1094,7 +1100,7 @@ struct RowSum {
 constexpr int kAccDepth = 4;
 constexpr size_t kAccSmem = size_t(kThreads / 32) * kAccDepth * 8 * kAsgRowBytes;
 
-template <bool values>
+template <bool values, bool wide>
 __global__ void __launch_bounds__(kThreads, 3) k_lloyd_accum(LloydArgs p) {
   extern __shared__ __align__(128) uint8_t acc_raw[];
   __shared__ int rows_s[kThreads / 32][kAccRowsPerWarp];   // positions of the rows to add
@@ -1126,14 +1132,22 @@ __global__ void __launch_bounds__(kThreads, 3) k_lloyd_accum(LloydArgs p) {
     __syncwarp();
     const uint32_t ring = smem_u32(acc_raw) + uint32_t(w * kAccDepth * 8 * kAsgRowBytes);
     const uint2* ringp = reinterpret_cast<const uint2*>(acc_raw + w * kAccDepth * 8 * kAsgRowBytes) + lane;
-    // rows 8b .. 8b + 7 into stage b % kAccDepth: half a warp per row
+    // rows 8b .. 8b + 7 into stage b % kAccDepth: half a warp per row (rows on
+    // an 8-byte boundary only, which keys and values may lie on: two copies a lane)
     auto issue = [&](int b) {
 #pragma unroll
       for (int q = 0; q < 8; q += 2) {
         const int x = 8 * b + q + (lane >> 4);
-        if (x < n)
-          cp_async16(ring + uint32_t(((b % kAccDepth) * 8 + q + (lane >> 4)) * kAsgRowBytes + (lane & 15) * 16),
-                     X + int64_t(rows[x]) * kHeadDim + 8 * (lane & 15), 16u);
+        if (x < n) {
+          const uint32_t dst = ring + uint32_t(((b % kAccDepth) * 8 + q + (lane >> 4)) * kAsgRowBytes + (lane & 15) * 16);
+          const __nv_bfloat16* src = X + int64_t(rows[x]) * kHeadDim + 8 * (lane & 15);
+          if constexpr (wide) {
+            cp_async16(dst, src, 16u);
+          } else {
+            cp_async8(dst, src);
+            cp_async8(dst + 8, src + 4);
+          }
+        }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
