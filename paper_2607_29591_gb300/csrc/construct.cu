@@ -495,7 +495,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       k_obs_pass2<<<dim3(ntiles, UL), kThreads, sm_obs2, stream>>>(oa);
       k_pool<<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(A, scores, s, UL, cfg.pool_kernel);
     } else {
-      k_score_keynorm<<<unsigned(cdiv(int64_t(US), 8)), 256, 0, stream>>>(K, scores, int64_t(US));
+      k_key_norms<true><<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(K, scores, knorm, int64_t(US));
     }
     RESKV_LAUNCH_CHECK("scoring");
     timing_ok &= timer.mark(kStRank);
@@ -595,7 +595,8 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     // read from a padded copy
     CUtensorMap tmK;
     if (rmax > 0) {
-      k_key_norm<<<unsigned(cdiv(int64_t(US), 8)), 256, 0, stream>>>(K, knorm, int64_t(US));
+      if (cfg.score_mode == RESKV_SCORE_OBS_POOL)         // (the query-free scores come with the norms)
+        k_key_norms<false><<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(K, nullptr, knorm, int64_t(US));
       if (kpad && cudaMemcpyAsync(kpad, K, US * kHeadDim * 2, cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
         return cleanup_fail(fail(RESKV_ERR_CUDA, "copying the keys"));
       if (!encode_key_tiles(&tmK, kpad ? kpad : K, std::max<uint64_t>(US, kTile)))

@@ -277,13 +277,16 @@ __global__ void k_pool(const float* A, double* scores, int64_t s, int UL, int po
 //
 // A bf16 value is M 2^e with an integer M < 2^8 (M = 128 + mantissa field for
 // normal values, the mantissa field for subnormals), so its square is
-// M^2 2^t with M^2 < 2^16 and t = 2e even, t in [-266, 242].  One warp per
-// row, four dims per lane.  With tmax the largest t of the row's nonzero
-// squares, every square with t >= tmax - 104 is an exact integer multiple of
-// 2^(tmax - 104) below 2^120, and 128 of them sum below 2^127: the warp adds
-// them as 128-bit integers and one lane rounds the sum.  A row with a
-// nonzero square below that window (its values span more than 52 binades)
-// goes to an exact 576-bit accumulator in one lane.
+// M^2 2^t with M^2 < 2^16 and t = 2e even, t in [-266, 242].  The common row
+// (k_key_norms): every nonzero value lies within 20 binades of the largest, so
+// all values are integers below 2^28 in units of the lowest of those binades,
+// their squares sum below 2^63 in 64-bit integers, one multiply-add each, and
+// one conversion rounds the sum.  Otherwise a warp takes the row
+// (keynorm_row): with tmax the largest t of the row's nonzero squares, every
+// square with t >= tmax - 104 is an exact integer multiple of 2^(tmax - 104)
+// below 2^120, and 128 of them sum below 2^127: it adds them as 128-bit
+// integers.  A row with a nonzero square below that window (its values span
+// more than 52 binades) goes to an exact 576-bit accumulator in one lane.
 
 using u128 = unsigned __int128;
 
@@ -341,12 +344,9 @@ __device__ double keynorm_wide(const __nv_bfloat16* rowp) {
   return a ? round_u128(a, (top - 3) * 32 - 266, sticky) : 0.0;
 }
 
-// One warp per row; the grid covers n_rows warps (blockDim a multiple of 32).
-__global__ void k_score_keynorm(const __nv_bfloat16* K, double* scores, int64_t n_rows) {
-  const int64_t row = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= n_rows) return;                              // whole warps leave together
-  const uint2 w = __ldg(reinterpret_cast<const uint2*>(K + row * kHeadDim) + lane);
+// The exact score of any row, by a whole warp; the result is valid in lane 0.
+__device__ __noinline__ double keynorm_row(const __nv_bfloat16* rowp, int lane) {
+  const uint2 w = __ldg(reinterpret_cast<const uint2*>(rowp) + lane);
   const uint32_t b[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
   uint32_t m2[4];
   int t[4];
@@ -370,20 +370,13 @@ __global__ void k_score_keynorm(const __nv_bfloat16* K, double* scores, int64_t 
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) scores[row] = acc;
-    return;
+    return acc;
   }
-  if (tmax == INT_MIN) {                                  // every value is zero
-    if (lane == 0) scores[row] = 0.0;
-    return;
-  }
+  if (tmax == INT_MIN) return 0.0;                        // every value is zero
   bool wide = false;
 #pragma unroll
   for (int j = 0; j < 4; ++j) wide |= m2[j] != 0 && t[j] < tmax - 104;
-  if (__any_sync(0xffffffffu, wide)) {
-    if (lane == 0) scores[row] = keynorm_wide(K + row * kHeadDim);
-    return;
-  }
+  if (__any_sync(0xffffffffu, wide)) return lane == 0 ? keynorm_wide(rowp) : 0.0;
   u128 a = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j)
@@ -394,7 +387,138 @@ __global__ void k_score_keynorm(const __nv_bfloat16* K, double* scores, int64_t 
     const uint64_t lo = __shfl_xor_sync(0xffffffffu, uint64_t(a), o);
     a += (u128(hi) << 64) | lo;
   }
-  if (lane == 0) scores[row] = round_u128(a, tmax - 104, false);
+  return lane == 0 ? round_u128(a, tmax - 104, false) : 0.0;
+}
+
+// the greater of two signed 16-bit halves each
+__device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("max.s16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+
+// 128 fp32 products summed in any order stay within 130 u of the sum, the root
+// and the product within 2 u each
+__device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.0f + 140.0f * 5.9604645e-8f); }
+
+// Per key row, in one read of the keys: with kScore the query-free score, and
+// (knorm not NULL) an upper bound of ||k|| for the Lloyd assignment's rounding
+// bound.  n_rows rows of 256 bytes.
+//
+// A warp takes 32 rows, four at a time with eight lanes each (two 16-byte loads
+// a lane, four rows' worth in flight; keys on an 8-byte boundary take 8-byte
+// loads), and every lane keeps the sum of one row,
+// so the conversion and the root are done once for 32 rows.  Memory bound in
+// principle (256 bytes a row); the integer sums issue about as long as the
+// loads take.  8.4M rows: 642 us for score and bound together, 2883 + 768 with a
+// warp per row and 128-bit sums; the bound alone, 2.1M rows: 77 us, 194.
+template <bool kScore>
+__global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restrict__ K, double* __restrict__ scores,
+                                                   float* __restrict__ knorm, int64_t n_rows) {
+  const int64_t base = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32;
+  if (base >= n_rows) return;                             // whole warps leave together
+  const int lane = threadIdx.x & 31, q = lane >> 3, c = lane & 7;
+  const bool wide = (reinterpret_cast<uintptr_t>(K) & 15u) == 0;
+  const int64_t mine = base + 4 * c + q;                  // the row whose sum this lane keeps
+  uint64_t sum = 0;                                       // kScore: in units of 2^(2 (e0 - 134))
+  float fsum = 0.f;
+  int e0 = 0;                                             // 0: not a common row
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    uint4 w[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t row = base + 4 * (4 * half + i) + q;
+      w[i][0] = w[i][1] = make_uint4(0, 0, 0, 0);
+      if (row < n_rows) {
+        const __nv_bfloat16* src = K + row * kHeadDim + 8 * c;
+        if (wide) {
+          w[i][0] = __ldg(reinterpret_cast<const uint4*>(src));
+          w[i][1] = __ldg(reinterpret_cast<const uint4*>(src) + 8);
+        } else {
+          const uint2* s8 = reinterpret_cast<const uint2*>(src);
+          const uint2 a = __ldg(s8), b = __ldg(s8 + 1), d = __ldg(s8 + 16), e = __ldg(s8 + 17);
+          w[i][0] = make_uint4(a.x, a.y, b.x, b.y);
+          w[i][1] = make_uint4(d.x, d.y, e.x, e.y);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t x[8] = {w[i][0].x, w[i][0].y, w[i][0].z, w[i][0].w,
+                             w[i][1].x, w[i][1].y, w[i][1].z, w[i][1].w};
+      if constexpr (kScore) {
+        // u: a value's bits without the sign.  The largest u, and the largest
+        // 2^15 - u of the nonzero values (a zero gives -2^15)
+        uint32_t big = 0, small = 0x80008000u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          big = max_s16x2(big, x[j] & 0x7fff7fffu);
+          small = max_s16x2(small, ~((x[j] | 0x80008000u) - 0x00010001u));
+        }
+        uint32_t mm = max_s16x2(__byte_perm(big, small, 0x5410), __byte_perm(big, small, 0x7632));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mm = max_s16x2(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+        const int emax = int(mm & 0xffffu) >> 7, umin = 0x8000 - (int(mm) >> 16);
+        const int elow = emax - 20;
+        uint64_t s64 = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+          for (int hw = 0; hw < 2; ++hw) {
+            const uint32_t u = hw ? x[j] >> 16 : x[j];
+            const int e = int((u >> 7) & 0xffu);
+            // 2^(e - elow) M: zero (all bits shifted out) below elow
+            uint32_t m;
+            asm("shl.b32 %0, %1, %2;" : "=r"(m) : "r"((u & 0x7fu) | 0x80u), "r"(e - elow));
+            s64 += uint64_t(m) * m;
+          }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s64 += __shfl_xor_sync(0xffffffffu, s64, o);
+        if (c == 4 * half + i) {
+          sum = s64;
+          e0 = elow >= 1 && emax != 0xff && umin >= (elow << 7) ? elow : 0;
+        }
+      } else {
+        float f = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float2 v = bf16x2_to_float2(x[j]);
+          f = fmaf(v.x, v.x, fmaf(v.y, v.y, f));
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        if (c == 4 * half + i) fsum = f;
+      }
+    }
+  }
+  if constexpr (!kScore) {
+    if (mine < n_rows) knorm[mine] = norm_bound(fsum);
+  } else {
+    if (mine < n_rows && e0) {
+      scores[mine] = __ull2double_rn(sum) * __hiloint2double((1023 + 2 * (e0 - 134)) << 20, 0);
+      if (knorm) {
+        const int E = e0 - 134;
+        const float unit = __uint_as_float(E >= -126 ? uint32_t(E + 127) << 23 : 1u << (E + 149));
+        const float nrm = __fmul_ru(norm_bound(__ull2float_ru(sum)), unit);
+        knorm[mine] = nrm < 1.8446744e19f ? nrm : INFINITY;        // as the fp32 sum: beyond 2^64 no bound
+      }
+    }
+    uint32_t rest = __ballot_sync(0xffffffffu, mine < n_rows && e0 == 0);
+    while (rest) {                                        // the other rows, one by one
+      const int l = __ffs(rest) - 1;
+      rest &= rest - 1;
+      const int64_t row = base + 4 * (l & 7) + (l >> 3);
+      const double sc = keynorm_row(K + row * kHeadDim, lane);
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(K + row * kHeadDim) + lane);
+      const float2 a = bf16x2_to_float2(v.x), b = bf16x2_to_float2(v.y);
+      const float f = warp_sum(fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y))));
+      if (lane == 0) {
+        scores[row] = sc;
+        if (knorm) knorm[row] = norm_bound(f);
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -269,21 +269,6 @@ __device__ __forceinline__ uint32_t push_sign(uint32_t m, float x) {
   return d;
 }
 
-// An upper bound of ||k|| for every key row (a warp per row), for the
-// assignment's bound: 128 fp32 products summed in any order stay within 130 u of
-// the sum, the root and the product within 2 u each.
-__global__ void k_key_norm(const __nv_bfloat16* __restrict__ K, float* __restrict__ out, int64_t rows) {
-  const int64_t row = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= rows) return;
-  const int lane = threadIdx.x & 31;
-  const uint2 w = *reinterpret_cast<const uint2*>(K + row * kHeadDim + 4 * lane);
-  const float2 a = bf16x2_to_float2(w.x), b = bf16x2_to_float2(w.y);
-  float s = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y)));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[row] = sqrtf(s) * (1.0f + 140.0f * 5.9604645e-8f);
-}
-
 // (unit, tile) of the flat tile order g = unit * ntiles + tile, stepped without
 // divisions, skipping units with no centre from seg0 on; r is read once per unit
 struct AsgCursor {
