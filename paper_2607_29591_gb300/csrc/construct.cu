@@ -332,6 +332,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   Scratch S;
   double* scores = nullptr;
   float* A = nullptr;
+  uint4* qfrag = nullptr;
   float2* tstats = nullptr;
   float2* rstats = nullptr;
   int32_t *top = nullptr, *rank_pos = nullptr, *assign = nullptr;
@@ -374,6 +375,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   if (adakv) S.get(&ada_counts, size_t(UL) * 2);
   if (n_fit_rows > 0) {
     S.get(&A, US);
+    S.get(&qfrag, size_t(UL) * cdiv(n_fit_rows, 16) * 256);
     S.get(&tstats, size_t(UL) * n_fit_rows * ntiles);
     S.get(&rstats, size_t(UL) * n_fit_rows);
   }
@@ -455,7 +457,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
 
   // kernel attributes
   const size_t sm_obs1 = size_t(kTile) * kAsgRowBytes;               // the key tile
-  const size_t sm_obs2 = sm_obs1 + size_t(kThreads / 32) * kTile * 4;  // + per-warp sums
+  const size_t sm_obs2 = sm_obs1 + size_t(8) * kTile * 4;  // + the partial sums
   // the ranked keys and positions, up to the next power of two of kTopThreads
   size_t n_sort = kTopThreads;
   while (n_sort < size_t(std::max(n_top, 1))) n_sort *= 2;
@@ -489,10 +491,11 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     // ---- token scores ----
     timing_ok &= timer.mark(kStScore);
     if (cfg.score_mode == RESKV_SCORE_OBS_POOL) {
-      ObsArgs oa{K, Q, s, G, cfg.n_obs, n_fit_rows, cfg.n_fit, ntiles, tstats, rstats, A};
-      k_obs_pass1<<<dim3(ntiles, UL), kThreads, sm_obs1, stream>>>(oa);
-      k_obs_rowstats<<<unsigned(cdiv(int64_t(UL) * n_fit_rows, 256)), 256, 0, stream>>>(oa, UL);
-      k_obs_pass2<<<dim3(ntiles, UL), kThreads, sm_obs2, stream>>>(oa);
+      ObsArgs oa{K, Q, s, G, cfg.n_obs, n_fit_rows, cfg.n_fit, ntiles, qfrag, tstats, rstats, A};
+      k_obs_frag<<<dim3(unsigned(cdiv(n_fit_rows, 16)), UL), 256, 0, stream>>>(oa);
+      k_obs_pass1<<<dim3(ntiles, UL), 32 * obs_warps1(n_fit_rows), sm_obs1, stream>>>(oa);
+      k_obs_rowstats<<<unsigned(cdiv(int64_t(UL) * n_fit_rows, 32)), 256, 0, stream>>>(oa, UL);
+      k_obs_pass2<<<dim3(ntiles, UL), 32 * obs_warps2(n_fit_rows), sm_obs2, stream>>>(oa);
       k_pool<<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(A, scores, s, UL, cfg.pool_kernel);
     } else {
       k_key_norms<true><<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(K, scores, knorm, int64_t(US));

@@ -75,184 +75,306 @@ struct ObsArgs {
   int32_t G, n_obs, n_rows;    // n_rows = G * n_fit, row = g * n_fit + t
   int32_t n_fit;
   int32_t ntiles;
+  uint4* qfrag;                // [UL, blocks of 16 rows, 8, 32] the fit rows as A fragments
   float2* tile_stats;          // [UL, n_rows, ntiles] (max, sum) per tile, log2 domain
   float2* row_stats;           // [UL, n_rows] (max, 1/sum)
   float* A;                    // [UL, s] attention summed over fit rows, averaged over G
 };
 
-// Logits of fit rows against a 128-token tile on the tensor cores: a warp
-// takes 16 query rows at a time (rows 16 rb .. 16 rb + 15, A fragments straight
-// from global memory), the keys are the B operand from the swizzled tile.
-// Products of the bf16 rows and keys are exact, accumulated in fp32, then
-// scaled by log2(e)/sqrt(d) (the logits in log2 units).  The accumulator of
-// n-tile nt holds rows g (entries 0, 1) and g + 8 (entries 2, 3) at tokens
-// 8 nt + 2 t4 (+1), with g = lane / 4, t4 = lane % 4.
-__device__ __forceinline__ const uint32_t* obs_row(const ObsArgs& p, int ul, int row) {
-  const int g = row / p.n_fit, t = row % p.n_fit;
-  return reinterpret_cast<const uint32_t*>(p.Qobs +
-                                           ((int64_t(ul) * p.G + g) * p.n_obs + t) * kHeadDim);
+// Logits of the fit rows against tiles of 128 keys on the tensor cores
+// (mma.sync m16n8k16): the queries are the A operand, 16 rows to a block, the
+// keys the B operand from the swizzled tile.  Products of the bf16 rows and keys
+// are exact, accumulated in fp32, then scaled by log2(e)/sqrt(d) (the logits in
+// log2 units).  The accumulator of n-tile nt holds rows g (entries 0, 1) and
+// g + 8 (entries 2, 3) at tokens 8 nt + 2 t4 (+1), with g = lane / 4,
+// t4 = lane % 4.
+//
+// What bounds it: reading fragments from shared memory and L1 (65 and 81 % of
+// the data pipe's wavefronts in the two passes, the tensor pipe 32 and 26 %, with
+// 16 rows per fragment of keys and the queries gathered row by row for every
+// tile).  So a warp takes two blocks of rows (32 rows) per fragment of keys, and
+// the queries come as whole fragments, laid out once per layer (k_obs_frag).  The
+// block has as many warps as there are row pairs to share evenly, and several
+// blocks per SM cover each other's loads.  64 units of 32K keys, 96 rows: passes
+// 361 + 472 us -> 204 + 252; 32 units of 128K keys, 384 rows: 2039 + 2579 ->
+// 1375 + 1273 (the tensor pipe, busy for about half of that, and the issue of the
+// exponentials between the products bound it now).
+__global__ void k_obs_frag(ObsArgs p) {          // grid (blocks of rows, UL), 256 threads
+  const int rb = blockIdx.x, ul = blockIdx.y;
+  const int ks = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+  auto row = [&](int r) -> const uint32_t* {
+    if (r >= p.n_rows) return nullptr;
+    const int h = r / p.n_fit, t = r % p.n_fit;
+    return reinterpret_cast<const uint32_t*>(p.Qobs + ((int64_t(ul) * p.G + h) * p.n_obs + t) * kHeadDim) + 8 * ks + t4;
+  };
+  const uint32_t *q0 = row(rb * 16 + g), *q1 = row(rb * 16 + g + 8);
+  p.qfrag[((int64_t(ul) * gridDim.x + rb) * 8 + ks) * 32 + lane] =
+      make_uint4(q0 ? __ldg(q0) : 0u, q1 ? __ldg(q1) : 0u, q0 ? __ldg(q0 + 4) : 0u, q1 ? __ldg(q1 + 4) : 0u);
 }
 
-__device__ __forceinline__ void obs_afrag(const ObsArgs& p, int ul, int rb, int lane,
-                                          uint32_t (&A)[8][4]) {
-  const int g = lane >> 2, t4 = lane & 3;
-  const int r0 = rb * 16 + g, r1 = r0 + 8;
-  const uint32_t* q0 = r0 < p.n_rows ? obs_row(p, ul, r0) : nullptr;
-  const uint32_t* q1 = r1 < p.n_rows ? obs_row(p, ul, r1) : nullptr;
+// the A fragments of row blocks rb and rb + 1 (zeros past the last block)
+__device__ __forceinline__ void obs_load_a(const ObsArgs& p, int ul, int rb, int nrb, int lane, uint4 (&A)[2][8]) {
+  const uint4* f = p.qfrag + (int64_t(ul) * nrb + rb) * 256 + lane;
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    A[ks][0] = q0 ? __ldg(q0 + 8 * ks + t4) : 0u;
-    A[ks][1] = q1 ? __ldg(q1 + 8 * ks + t4) : 0u;
-    A[ks][2] = q0 ? __ldg(q0 + 8 * ks + 4 + t4) : 0u;
-    A[ks][3] = q1 ? __ldg(q1 + 8 * ks + 4 + t4) : 0u;
-  }
+  for (int ks = 0; ks < 8; ++ks) A[0][ks] = __ldg(f + 32 * ks);
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks) A[1][ks] = rb + 1 < nrb ? __ldg(f + 256 + 32 * ks) : make_uint4(0, 0, 0, 0);
 }
 
-// logits of the 16 rows against tokens 64 h .. 64 h + 63 of the tile
-__device__ __forceinline__ void obs_half_logits(uint32_t ks_s, int h, int lane,
-                                                const uint32_t (&A)[8][4], float (&S)[8][4]) {
+// logits of the (one or) two row blocks against tokens tk .. tk + 16 NP - 1 of the tile
+template <int NP>
+__device__ __forceinline__ void obs_logits(uint32_t ks_s, int tk, int lane, const uint4 (&A)[2][8], bool two,
+                                           float (&S)[2][2 * NP][4]) {
   const int mi = lane >> 3;
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt) S[nt][0] = S[nt][1] = S[nt][2] = S[nt][3] = 0.f;
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-  for (int np = 0; np < 4; ++np) {
-    const int trow = 64 * h + 16 * np + (mi >> 1) * 8 + (lane & 7);
+    for (int nt = 0; nt < 2 * NP; ++nt) S[i][nt][0] = S[i][nt][1] = S[i][nt][2] = S[i][nt][3] = 0.f;
+  const int trow = tk + (mi >> 1) * 8 + (lane & 7);
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
+  for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+    for (int np = 0; np < NP; ++np) {
       uint32_t b0, b1, b2, b3;
-      ldsm_x4(ks_s + asg_swz(trow, 2 * ks + (mi & 1)), b0, b1, b2, b3);
-      mma16816(S[2 * np], A[ks][0], A[ks][1], A[ks][2], A[ks][3], b0, b1);
-      mma16816(S[2 * np + 1], A[ks][0], A[ks][1], A[ks][2], A[ks][3], b2, b3);
+      ldsm_x4(ks_s + asg_swz(trow + 16 * np, 2 * ks + (mi & 1)), b0, b1, b2, b3);
+      mma16816(S[0][2 * np], A[0][ks].x, A[0][ks].y, A[0][ks].z, A[0][ks].w, b0, b1);
+      mma16816(S[0][2 * np + 1], A[0][ks].x, A[0][ks].y, A[0][ks].z, A[0][ks].w, b2, b3);
+      if (two) {
+        mma16816(S[1][2 * np], A[1][ks].x, A[1][ks].y, A[1][ks].z, A[1][ks].w, b0, b1);
+        mma16816(S[1][2 * np + 1], A[1][ks].x, A[1][ks].y, A[1][ks].z, A[1][ks].w, b2, b3);
+      }
     }
-  }
   const float scale = kLog2e * rsqrtf(float(kHeadDim));
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int nt = 0; nt < 2 * NP; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) S[i][nt][e] *= scale;
+}
+
+// Warps of a block of the first pass: one per pair of row blocks where there are
+// few, else the count of 4, 3 or 6 that leaves the fewest idle in the last round.
+__host__ inline int obs_warps1(int n_rows) {
+  const int pairs = ((n_rows + 15) / 16 + 1) / 2;
+  if (pairs <= 3) return pairs;
+  int best = 4;
+  for (int w : {3, 6})
+    if ((pairs + w - 1) / w * w < (pairs + best - 1) / best * best) best = w;
+  return best;
+}
+// of the second: its items are (pair of partial sums, half of the tile)
+__host__ inline int obs_warps2(int n_rows) {
+  const int pairs = (std::min((n_rows + 15) / 16, 8) + 1) / 2;
+  return pairs <= 2 ? 2 * pairs : pairs;
+}
+
+// (max, sum) of one row's 16 logits of this lane and its three neighbours'
+// (64 tokens), folded into the row's; n tokens of the half exist
+template <bool ragged>
+__device__ __forceinline__ void obs_fold(const float (&S)[8][4], int a, int t4, int n, float& M, float& L) {
+  float mx = -INFINITY;
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) S[nt][e] *= scale;
+    for (int c = 0; c < 2; ++c)
+      if (!ragged || 8 * nt + 2 * t4 + c < n) mx = fmaxf(mx, S[nt][2 * a + c]);
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  float sum = 0.f;
+  if (mx != -INFINITY) {
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        if (!ragged || 8 * nt + 2 * t4 + c < n) sum += exp2f(S[nt][2 * a + c] - mx);
+  }
+  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  if (mx != -INFINITY) {
+    const float nm = fmaxf(M, mx);
+    L = L * exp2f(M - nm) + sum * exp2f(mx - nm);
+    M = nm;
+  }
 }
 
 // Pass 1: per (row, tile) max and sum of 2^{a log2e} over the tile's tokens.
-__global__ void __launch_bounds__(kThreads, 2) k_obs_pass1(ObsArgs p) {
+__global__ void __launch_bounds__(192, 2) k_obs_pass1(ObsArgs p) {
   extern __shared__ __align__(128) uint8_t obs_raw[];
   const int tile = blockIdx.x, ul = blockIdx.y;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
   const int64_t tok0 = int64_t(tile) * kTile;
   const uint32_t ks_s = smem_u32(obs_raw);
   stage_key_tile(ks_s, p.K + int64_t(ul) * p.s * kHeadDim, p.s, tok0);
+  const int nrb = (p.n_rows + 15) / 16, n_tok = int(min(int64_t(kTile), p.s - tok0));
+  uint4 A[2][8];
+  obs_load_a(p, ul, 2 * w, nrb, lane, A);        // (every warp has a pair)
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  for (int rb = w; rb * 16 < p.n_rows; rb += kThreads / 32) {
-    uint32_t A[8][4];
-    obs_afrag(p, ul, rb, lane, A);
-    float M[2] = {-INFINITY, -INFINITY}, Lsum[2] = {0.f, 0.f};    // rows g, g + 8
+  for (int rb = 2 * w; rb < nrb;) {
+    const bool two = rb + 1 < nrb;
+    float M[2][2], L[2][2];                      // rows g, g + 8 of the two blocks
 #pragma unroll
+    for (int i = 0; i < 2; ++i) M[i][0] = M[i][1] = -INFINITY, L[i][0] = L[i][1] = 0.f;
+#pragma unroll 1
     for (int h = 0; h < 2; ++h) {
-      float S[8][4];
-      obs_half_logits(ks_s, h, lane, A, S);
+      float S[2][8][4];
+      obs_logits<4>(ks_s, 64 * h, lane, A, two, S);
+      const int n = n_tok - 64 * h;
+      if (n >= 64) {
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        float mx = -INFINITY;
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
+          for (int a = 0; a < 2; ++a) obs_fold<false>(S[i], a, t4, n, M[i][a], L[i][a]);
+      } else {
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
-            if (tok0 + 64 * h + 8 * nt + 2 * t4 + c < p.s) mx = fmaxf(mx, S[nt][2 * a + c]);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        float sum = 0.f;
-        if (mx != -INFINITY) {
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-              if (tok0 + 64 * h + 8 * nt + 2 * t4 + c < p.s) sum += exp2f(S[nt][2 * a + c] - mx);
-        }
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        if (mx != -INFINITY) {                    // fold the half into the row's (max, sum)
-          const float nm = fmaxf(M[a], mx);
-          Lsum[a] = Lsum[a] * exp2f(M[a] - nm) + sum * exp2f(mx - nm);
-          M[a] = nm;
-        }
+          for (int a = 0; a < 2; ++a) obs_fold<true>(S[i], a, t4, n, M[i][a], L[i][a]);
       }
     }
     if (t4 == 0) {
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int row = rb * 16 + g + 8 * a;
-        if (row < p.n_rows)
-          p.tile_stats[(int64_t(ul) * p.n_rows + row) * p.ntiles + tile] =
-              make_float2(M[a], Lsum[a]);
-      }
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const int row = (rb + i) * 16 + g + 8 * a;
+          if (row < p.n_rows)
+            p.tile_stats[(int64_t(ul) * p.n_rows + row) * p.ntiles + tile] = make_float2(M[i][a], L[i][a]);
+        }
     }
+    rb += 2 * (blockDim.x >> 5);
+    if (rb < nrb) obs_load_a(p, ul, rb, nrb, lane, A);
   }
 }
 
-// Row statistics over all tiles (in tile order).
-__global__ void k_obs_rowstats(ObsArgs p, int UL) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= int64_t(UL) * p.n_rows) return;
-  const float2* t = p.tile_stats + i * p.ntiles;
+// Row statistics over all tiles: the sums in tile order, one chain of fused
+// multiply-adds per row.  32 rows per block of 256 threads: the maxima and the
+// exponentials take eight threads a row, the chains a lane each, one chunk of
+// tiles behind.  Latency bound (the chain: 4 cycles a tile); 3072 rows of 256
+// tiles: 9 us, 99 with the loads and exponentials in the chain too.
+constexpr int kStatChunk = 64;
+
+__global__ void __launch_bounds__(256) k_obs_rowstats(ObsArgs p, int UL) {
+  __shared__ float2 term[2][32][kStatChunk + 1];
+  const int64_t n = int64_t(UL) * p.n_rows, row0 = int64_t(blockIdx.x) * 32;
+  const int rl = threadIdx.x >> 3, sub = threadIdx.x & 7, lane = threadIdx.x & 31;
+  const bool in = row0 + rl < n;
+  const float2* t = p.tile_stats + (row0 + rl) * p.ntiles;
   float mx = -INFINITY;
-  for (int k = 0; k < p.ntiles; ++k) mx = fmaxf(mx, t[k].x);
+  if (in)
+    for (int k = sub; k < p.ntiles; k += 8) mx = fmaxf(mx, t[k].x);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const int nch = (p.ntiles + kStatChunk - 1) / kStatChunk;
   float sum = 0.f;
-  for (int k = 0; k < p.ntiles; ++k)
-    if (t[k].y > 0.f) sum += t[k].y * exp2f(t[k].x - mx);
-  p.row_stats[i] = make_float2(mx, 1.0f / sum);
+  for (int c = 0; c <= nch; ++c) {
+    if (c < nch && in) {
+#pragma unroll
+      for (int j = 0; j < kStatChunk / 8; ++j) {
+        const int k = c * kStatChunk + sub + 8 * j;
+        const float2 v = k < p.ntiles ? t[k] : make_float2(0.f, 0.f);
+        term[c & 1][rl][sub + 8 * j] = v.y > 0.f ? make_float2(v.y, exp2f(v.x - mx)) : make_float2(0.f, 0.f);
+      }
+    }
+    if (c > 0 && threadIdx.x < 32) {
+      const float2* v = term[(c - 1) & 1][lane];
+#pragma unroll 16
+      for (int k = 0; k < kStatChunk; ++k) sum += v[k].x * v[k].y;
+    }
+    __syncthreads();
+  }
+  // the row's maximum lies with its eight threads, its sum with lane `row` of warp 0
+  float* m_s = reinterpret_cast<float*>(term);
+  if (sub == 0) m_s[rl] = mx;
+  __syncthreads();
+  if (threadIdx.x < 32 && row0 + lane < n) p.row_stats[row0 + lane] = make_float2(m_s[lane], 1.0f / sum);
 }
 
-// Pass 2: A_p = (1/G) sum over fit rows of the softmax weight of token p.
-__global__ void __launch_bounds__(kThreads, 2) k_obs_pass2(ObsArgs p) {
+// the softmax weights of two row blocks, added to this lane's column sums of the
+// 64 tokens from tk on; all: every row has a finite positive sum
+template <bool all>
+__device__ __forceinline__ void obs_columns(uint32_t ks_s, int tk, int lane, const uint4 (&A)[2][8], bool two,
+                                            const float2 (&st)[2][2], float (&col)[2][8][2]) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {                  // 32 tokens at a time
+    float S[2][4][4];
+    obs_logits<2>(ks_s, tk + 32 * q, lane, A, two, S);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int a = 0; a < 2; ++a)
+            if (all || st[i][a].y > 0.f) col[i][4 * q + nt][c] += exp2f(S[i][nt][2 * a + c] - st[i][a].x) * st[i][a].y;
+  }
+}
+
+// Pass 2: A_p = (1/G) sum over fit rows of the softmax weight of token p.  The
+// sums are formed apart for the row blocks congruent mod 8, in ascending order,
+// and added in the order of the remainders: a warp takes two remainders and half
+// of the tile's tokens.
+__global__ void __launch_bounds__(128, 3) k_obs_pass2(ObsArgs p) {
   extern __shared__ __align__(128) uint8_t obs_raw[];
-  float* red = reinterpret_cast<float*>(obs_raw + kTile * kAsgRowBytes);   // [8 warps][128 tokens]
+  float* red = reinterpret_cast<float*>(obs_raw + kTile * kAsgRowBytes);   // [8 remainders][128 tokens]
   const int tile = blockIdx.x, ul = blockIdx.y;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
   const int64_t tok0 = int64_t(tile) * kTile;
   const uint32_t ks_s = smem_u32(obs_raw);
   stage_key_tile(ks_s, p.K + int64_t(ul) * p.s * kHeadDim, p.s, tok0);
+  const int nrb = (p.n_rows + 15) / 16, n_rem = min(nrb, 8), pairs = (n_rem + 1) / 2;
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  for (int h = 0; h < 2; ++h) {                  // tokens 64 h .. 64 h + 63
-    float col[8][2];                             // this lane's column sums
+  for (int it = w; it < 2 * pairs; it += blockDim.x >> 5) {
+    // with four pairs: the first two, which may have a block of rows more, share
+    // the first round
+    const int pr = pairs == 4 ? 2 * (it >> 2) + (it & 1) : it % pairs, h = pairs == 4 ? (it >> 1) & 1 : it / pairs;
+    float col[2][8][2];                          // this lane's column sums
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) col[nt][0] = col[nt][1] = 0.f;
-    for (int rb = w; rb * 16 < p.n_rows; rb += kThreads / 32) {
-      uint32_t A[8][4];
-      obs_afrag(p, ul, rb, lane, A);
-      float2 st[2];
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int row = rb * 16 + g + 8 * a;
-        st[a] = row < p.n_rows ? p.row_stats[int64_t(ul) * p.n_rows + row] : make_float2(0.f, 0.f);
+      for (int nt = 0; nt < 8; ++nt) col[i][nt][0] = col[i][nt][1] = 0.f;
+#pragma unroll 1
+    for (int rb = 2 * pr; rb < nrb; rb += 8) {
+      const bool two = rb + 1 < nrb;
+      uint4 A[2][8];
+      obs_load_a(p, ul, rb, nrb, lane, A);
+      float2 st[2][2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const int row = (rb + i) * 16 + g + 8 * a;
+          st[i][a] = row < p.n_rows ? p.row_stats[int64_t(ul) * p.n_rows + row] : make_float2(0.f, 0.f);
+        }
+      const bool all = __all_sync(0xffffffffu, st[0][0].y > 0.f && st[0][1].y > 0.f && st[1][0].y > 0.f && st[1][1].y > 0.f);
+      if (all) {
+        obs_columns<true>(ks_s, 64 * h, lane, A, true, st, col);
+      } else {                                   // rows past the last, or without a finite sum
+        obs_columns<false>(ks_s, 64 * h, lane, A, two, st, col);
       }
-      float S[8][4];
-      obs_half_logits(ks_s, h, lane, A, S);
+    }
+    // sum over the eight row groups of the warp (the remainders are summed below)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-          for (int a = 0; a < 2; ++a)
-            if (st[a].y > 0.f) col[nt][c] += exp2f(S[nt][2 * a + c] - st[a].x) * st[a].y;
-    }
-    // sum over the eight row groups of the warp (the warps are summed below)
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float v = col[nt][c];
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v += __shfl_xor_sync(0xffffffffu, v, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        if (g == 0) red[w * kTile + 64 * h + 8 * nt + 2 * t4 + c] = v;
-      }
+        for (int c = 0; c < 2; ++c) {
+          float v = col[i][nt][c];
+          v += __shfl_xor_sync(0xffffffffu, v, 4);
+          v += __shfl_xor_sync(0xffffffffu, v, 8);
+          v += __shfl_xor_sync(0xffffffffu, v, 16);
+          if (g == 0) red[(2 * pr + i) * kTile + 64 * h + 8 * nt + 2 * t4 + c] = v;
+        }
   }
   __syncthreads();
-  if (threadIdx.x < kTile) {
+  for (int i = threadIdx.x; i < kTile; i += blockDim.x) {
     float a = 0.f;
-    for (int ww = 0; ww < kThreads / 32; ++ww) a += red[ww * kTile + threadIdx.x];
-    const int64_t tok = tok0 + threadIdx.x;
+    for (int rem = 0; rem < n_rem; ++rem) a += red[rem * kTile + i];
+    const int64_t tok = tok0 + i;
     if (tok < p.s) p.A[int64_t(ul) * p.s + tok] = a / float(p.G);
   }
 }
