@@ -640,7 +640,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
               la, sg * segw, segw, lloyd_asg_key_bufs(segw), tmK);
           la.test_fault = 0;
         }
-        k_lloyd_resolve<<<unsigned(4 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
+        k_lloyd_resolve<<<unsigned(3 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
         k_lloyd_scatter<false><<<gs, kScatterThreads, size_t(r_hi) * 4 * sizeof(int), stream>>>(la);
         (k16 ? k_lloyd_accum<false, true> : k_lloyd_accum<false, false>)<<<ga, kThreads, kAccSmem, stream>>>(la);
         if (last) {                       // the values of every member

@@ -684,9 +684,17 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
   }
 }
 
-// The decision of the tokens k_lloyd_assign left, a warp per token (lane l
-// holds dims 4l..4l+3).  Candidates: the two kept centres, or every centre when
-// more were within the tensor-core bound.
+// The decision of the tokens k_lloyd_assign left.  Candidates: the two kept
+// centres (nearly always), or every centre when more were within the tensor-core
+// bound.  A warp takes four tokens of two candidates at once, eight lanes each
+// (lane l on dims 4l + 32i .. 4l + 32i + 3, i < 4).  The tokens of all centres
+// that the CTA met are queued and their distances shared out over its warps (lane
+// l on dims 4l .. 4l + 3), then a warp per token decides.  A distance is the same
+// tree of sums either way: chains of 4 dims, then dims 64, 32, 16, 8 and 4 apart.
+// Bound by latency: 0.3 to 0.9 % of the tokens come here, one in a hundred of them
+// with all centres, whose serial scan by one warp used to end the kernel.  64
+// units of 32K keys, r = 51 .. 205: 18 us on average, 34 with a warp per token of
+// either kind; 32 units of 128K keys, r = 102 .. 410: 34, 67.
 //
 // First their distances are taken directly in fp32, d32_j = sum_i (k_i -
 // c32_i)^2 against the fp32 centres: no cancellation, so the error is small
@@ -702,9 +710,11 @@ constexpr int kResWarps = 8;
 constexpr int kResChunk = 256;                  // distances held at once
 constexpr int kResMaxCtas = 1024;               // assignment CTAs (one list each)
 
-__global__ void __launch_bounds__(kResWarps * 32) k_lloyd_resolve(LloydArgs p, int n_lists) {
-  __shared__ float dsm[kResWarps][kResChunk];     // candidate distances (fp32)
+__global__ void __launch_bounds__(kResWarps * 32, 3) k_lloyd_resolve(LloydArgs p, int n_lists) {
+  __shared__ float dsm[kResWarps][kResChunk];     // candidate distances (fp32) of kResWarps queued tokens
   __shared__ int jsm[kResWarps][kResChunk];       // centres left for fp64
+  __shared__ int2 queue[4 * kResWarps];           // (unit, position) of the tokens of all centres
+  __shared__ int queued;
   __shared__ int pre[kResMaxCtas + 1];            // tokens in the lists before list i
   __shared__ int warp_sums[32];
   const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
@@ -720,155 +730,267 @@ __global__ void __launch_bounds__(kResWarps * 32) k_lloyd_resolve(LloydArgs p, i
       pre[i] = run;
       run += p.amb_count[i];
     }
-    if (threadIdx.x == 0) pre[n_lists] = total;
+    if (threadIdx.x == 0) {
+      pre[n_lists] = total;
+      queued = 0;
+    }
     __syncthreads();
   }
   const int n = pre[n_lists];
   const int64_t n_all = int64_t(p.n_units) * p.ntiles;
   const int nw = int((int64_t(gridDim.x) * blockDim.x) >> 5);
   const float uu = 5.9604645e-8f;
-  for (int i = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5); i < n; i += nw) {
-    int li = 0, hi_l = n_lists;                   // the list holding token i
-    while (hi_l - li > 1) {
-      const int mid = (li + hi_l) >> 1;
-      if (pre[mid] <= i) li = mid;
-      else hi_l = mid;
+  // the decision res (>= r: none, only NaN distances get there)
+  auto settle = [&](int u, int r, int64_t pos, int res) {
+    if (res >= r) {
+      report_status(p.status, kStatusBadIndex);
+      res = 0;
     }
-    const int4 e = p.amb[(n_all * li / n_lists) * kTile + (i - pre[li])];
-    const int u = e.x, r = p.r_unit[u], ul = u % p.UL;
-    const int64_t pos = e.y;
-    const bool fs = e.z < 0;
-    const int js0 = e.z & 0x7fffffff, js1 = e.w;
-    const int nc_all = fs ? r : 2;
-    auto cand = [&](int k) { return fs ? k : (k == 0 ? js0 : js1); };
-    const uint2 kw = *reinterpret_cast<const uint2*>(p.K + (int64_t(ul) * p.s + pos) * kHeadDim + 4 * lane);
-    const float2 k01 = bf16x2_to_float2(kw.x), k23 = bf16x2_to_float2(kw.y);
-    const float* c32 = p.centers32 + int64_t(u) * p.rmax * kHeadDim + 4 * lane;
-    const float* cnu = p.cnorm + int64_t(u) * p.rmax;
-    auto bound = [&](float d, int j) {
-      const float cn = sqrtf(cnu[j]) * 1.001f;
-      return 16.0f * uu * d + 3.0f * uu * cn * (sqrtf(d) + uu * cn);
-    };
-    const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
-    float bd = INFINITY, hi = INFINITY;             // the fp32 best, the upper end of its interval
-    int bj = INT_MAX, na = 0;                       // its index; centres that may be nearest
-    bool over = false;                              // more of them than jl holds
-    for (int kc = 0; kc < nc_all; kc += kResChunk) {
-      const int nc = min(kResChunk, nc_all - kc);
-      // fp32 distances, eight centres at a time: a 4-term chain per lane, then
-      // a transposed butterfly (9 shuffles) that leaves centre 4 b4 + 2 b3 + b2
-      // (b_i: bit i of the lane) summed over all lanes -- five levels of adds,
-      // as the bound assumes
-      for (int k0 = 0; k0 < nc; k0 += 8) {
-        float a[8];
+    p.assign[int64_t(u) * p.s + pos] = res;
+    const int old = p.assign_prev ? p.assign_prev[int64_t(u) * p.s + pos] : -1;
+    if (res != old) {
+      atomicAdd(p.mcount + 2 * int64_t(u) * p.rmax + res, 1);
+      if (old >= 0) atomicAdd(p.mcount + (2 * int64_t(u) + 1) * p.rmax + min(old, r - 1), 1);
+    }
+  };
+  auto interval = [&](float d, float norm2) {
+    const float cn = sqrtf(norm2) * 1.001f;
+    return 16.0f * uu * d + 3.0f * uu * cn * (sqrtf(d) + uu * cn);
+  };
+  // (four tokens nw apart: where there are few, every warp has one at most)
+  for (int64_t i0 = 0; i0 < n; i0 += 4 * nw) {
+    const int64_t i = i0 + ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) + int64_t(lane >> 3) * nw;
+    const int c8 = lane & 7;
+    int4 e = make_int4(0, 0, 0, 0);
+    if (i < n) {
+      int li = 0, hi_l = n_lists;                 // the list holding token i
+      while (hi_l - li > 1) {
+        const int mid = (li + hi_l) >> 1;
+        if (pre[mid] <= i) li = mid;
+        else hi_l = mid;
+      }
+      e = p.amb[(n_all * li / n_lists) * kTile + (i - pre[li])];
+    }
+    const bool pair = i < n && e.z >= 0;
+    if (pair) {
+      const int u = e.x, r = p.r_unit[u];
+      const int64_t pos = e.y;
+      const int j2[2] = {e.z, e.w};
+      const __nv_bfloat16* krow = p.K + (int64_t(u % p.UL) * p.s + pos) * kHeadDim + 4 * c8;
+      const unsigned group = 0xffu << (lane & 24);
+      uint2 kw[4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int k = kc + (k0 + q < nc ? k0 + q : k0);
-          const float4 c = *reinterpret_cast<const float4*>(c32 + int64_t(cand(k)) * kHeadDim);
-          const float x0 = k01.x - c.x, x1 = k01.y - c.y, x2 = k23.x - c.z, x3 = k23.y - c.w;
+      for (int q = 0; q < 4; ++q) kw[q] = *reinterpret_cast<const uint2*>(krow + 32 * q);
+      float d2[2], nn[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float* c = p.centers32 + (int64_t(u) * p.rmax + j2[k]) * kHeadDim + 4 * c8;
+        nn[k] = p.cnorm[int64_t(u) * p.rmax + j2[k]];
+        float a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 v = *reinterpret_cast<const float4*>(c + 32 * q);
+          const float2 k01 = bf16x2_to_float2(kw[q].x), k23 = bf16x2_to_float2(kw[q].y);
+          const float x0 = k01.x - v.x, x1 = k01.y - v.y, x2 = k23.x - v.z, x3 = k23.y - v.w;
           a[q] = fmaf(x3, x3, fmaf(x2, x2, fmaf(x1, x1, x0 * x0)));
         }
-        float bq[4], cq[2];
-#pragma unroll
-        for (int i2 = 0; i2 < 4; ++i2) {
-          const float send = b4 ? a[i2] : a[i2 + 4];
-          bq[i2] = (b4 ? a[i2 + 4] : a[i2]) + __shfl_xor_sync(0xffffffffu, send, 16);
-        }
-#pragma unroll
-        for (int i2 = 0; i2 < 2; ++i2) {
-          const float send = b3 ? bq[i2] : bq[i2 + 2];
-          cq[i2] = (b3 ? bq[i2 + 2] : bq[i2]) + __shfl_xor_sync(0xffffffffu, send, 8);
-        }
-        float dq = (b2 ? cq[1] : cq[0]) + __shfl_xor_sync(0xffffffffu, b2 ? cq[0] : cq[1], 4);
-        dq += __shfl_xor_sync(0xffffffffu, dq, 2);
-        dq += __shfl_xor_sync(0xffffffffu, dq, 1);
-        const int v = 4 * b4 + 2 * b3 + b2;
-        if ((lane & 3) == 0 && k0 + v < nc) dl[k0 + v] = dq;
-      }
-      __syncwarp();
-      // the fp32 best (distance, index)
-      for (int k = lane; k < nc; k += 32) {
-        const float d = dl[k];
-        const int j = cand(kc + k);
-        if (d < bd || (d == bd && j < bj)) {
-          bd = d;
-          bj = j;
-        }
+        d2[k] = (a[0] + a[2]) + (a[1] + a[3]);
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        if (od < bd || (od == bd && oj < bj)) {
-          bd = od;
-          bj = oj;
+      for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) d2[k] += __shfl_xor_sync(group, d2[k], o);
+      float bd = INFINITY, bn = 0.f;              // the fp32 best, its centre's norm and index
+      int bj = INT_MAX, na = 0;                   // (and how many may be nearest)
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (d2[k] < bd || (d2[k] == bd && j2[k] < bj)) {
+          bd = d2[k];
+          bn = nn[k];
+          bj = j2[k];
         }
-      }
-      // the centres of the chunk whose interval reaches the best's so far
-      if (bj < r) hi = bd + bound(bd, bj);
-      for (int k0 = 0; k0 < nc; k0 += 32) {
-        const int k = k0 + lane;
-        bool m = false;
-        if (k < nc) {
-          const float d = dl[k];
-          m = !(d - bound(d, cand(kc + k)) > hi);
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, m);
-        if (na + __popc(bal) > kResChunk) over = true;
-        else if (m) jl[na + __popc(bal & ((1u << lane) - 1u))] = cand(kc + k);
-        if (!over) na += __popc(bal);
-      }
-      __syncwarp();
-    }
-    int res = bj;
-    if (bj < r && (na > 1 || over)) {               // fp64 decides among them
-      const double kx[4] = {k01.x, k01.y, k23.x, k23.y};
-      const double* c64 = p.centers64 + int64_t(u) * p.rmax * kHeadDim + 4 * lane;
-      double bd64 = INFINITY;
-      int bj64 = INT_MAX;
-      const int nq = over ? nc_all : na;
-      for (int k0 = 0; k0 < nq; k0 += 4) {
-        int jq[4];
+      const float hi = bj < r ? bd + interval(bd, bn) : INFINITY;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) jq[q] = k0 + q < nq ? (over ? cand(k0 + q) : jl[k0 + q]) : -1;
-        double a[4];
+      for (int k = 0; k < 2; ++k) na += !(d2[k] - interval(d2[k], nn[k]) > hi);
+      int res = bj;
+      if (bj < r && na > 1) {                     // fp64 decides
+        double bd64 = INFINITY;
+        res = INT_MAX;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const double4_32a c =
-              *reinterpret_cast<const double4_32a*>(c64 + int64_t(jq[q] < 0 ? 0 : jq[q]) * kHeadDim);
-          double tt = (kx[0] - c.x) * (kx[0] - c.x);
-          tt = fma(kx[1] - c.y, kx[1] - c.y, tt);
-          tt = fma(kx[2] - c.z, kx[2] - c.z, tt);
-          a[q] = fma(kx[3] - c.w, kx[3] - c.w, tt);
-        }
+        for (int k = 0; k < 2; ++k) {
+          const double* c = p.centers64 + (int64_t(u) * p.rmax + j2[k]) * kHeadDim + 4 * c8;
+          double a[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+          for (int q = 0; q < 4; ++q) {
+            const double4_32a v = *reinterpret_cast<const double4_32a*>(c + 32 * q);
+            const float2 k01 = bf16x2_to_float2(kw[q].x), k23 = bf16x2_to_float2(kw[q].y);
+            const double kx[4] = {k01.x, k01.y, k23.x, k23.y};
+            double tt = (kx[0] - v.x) * (kx[0] - v.x);
+            tt = fma(kx[1] - v.y, kx[1] - v.y, tt);
+            tt = fma(kx[2] - v.z, kx[2] - v.z, tt);
+            a[q] = fma(kx[3] - v.w, kx[3] - v.w, tt);
+          }
+          double dd = (a[0] + a[2]) + (a[1] + a[3]);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const double dd = __shfl_sync(0xffffffffu, a[q], 0);
-          if (jq[q] >= 0 && (dd < bd64 || (dd == bd64 && jq[q] < bj64))) {
+          for (int o = 4; o > 0; o >>= 1) dd += __shfl_xor_sync(group, dd, o);
+          if (dd < bd64 || (dd == bd64 && j2[k] < res)) {
             bd64 = dd;
-            bj64 = jq[q];
+            res = j2[k];
           }
         }
       }
-      res = bj64;
+      if (c8 == 0) settle(u, r, pos, res);
     }
-    if (lane == 0) {
-      if (res >= r) {                                   // only NaN distances get here
-        report_status(p.status, kStatusBadIndex);
-        res = 0;
+    // tokens of all centres
+    if (c8 == 0 && i < n && !pair) queue[atomicAdd(&queued, 1)] = make_int2(e.x, e.y);
+    __syncthreads();
+    const int m = queued;
+    for (int t0 = 0; t0 < m; t0 += kResWarps) {
+      const int mb = min(kResWarps, m - t0);
+      int r_hi = 0;
+      for (int t = 0; t < mb; ++t) r_hi = max(r_hi, p.r_unit[queue[t0 + t].x]);
+      const bool mine = wb < mb;                        // the token this warp decides
+      const int2 tok = queue[t0 + (mine ? wb : 0)];
+      const int r = p.r_unit[tok.x];
+      const float* cnu = p.cnorm + int64_t(tok.x) * p.rmax;
+      auto bound = [&](float d, int j) { return interval(d, cnu[j]); };
+      auto key = [&](int2 t, float2& k01, float2& k23) {
+        const uint2 kw = *reinterpret_cast<const uint2*>(p.K + (int64_t(t.x % p.UL) * p.s + t.y) * kHeadDim + 4 * lane);
+        k01 = bf16x2_to_float2(kw.x);
+        k23 = bf16x2_to_float2(kw.y);
+      };
+      const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
+      float bd = INFINITY, hi = INFINITY;               // the fp32 best, the upper end of its interval
+      int bj = INT_MAX, na = 0;                         // its index; centres that may be nearest
+      bool over = false;                                // more of them than jl holds
+      for (int kc = 0; kc < r_hi; kc += kResChunk) {
+        // fp32 distances: a 4-term chain per lane, then for each eight centres a
+        // transposed butterfly (9 shuffles) that leaves centre 4 b4 + 2 b3 + b2
+        // (b_i: bit i of the lane) summed over all lanes -- five levels of adds,
+        // as the bound assumes
+        constexpr int kOct = 2;
+        const int steps = (min(kResChunk, r_hi - kc) + 8 * kOct - 1) / (8 * kOct);
+        for (int x = wb; x < mb * steps; x += kResWarps) {
+          const int t = x % mb, k0 = x / mb * 8 * kOct;
+          const int2 tk = queue[t0 + t];
+          const int nc = min(kResChunk, p.r_unit[tk.x] - kc);
+          if (k0 >= nc) continue;
+          const float* c32 = p.centers32 + (int64_t(tk.x) * p.rmax + kc) * kHeadDim + 4 * lane;
+          float2 k01, k23;
+          key(tk, k01, k23);
+          float4 c[kOct][8];
+#pragma unroll
+          for (int h = 0; h < kOct; ++h)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int k = k0 + 8 * h + q;
+              c[h][q] = *reinterpret_cast<const float4*>(c32 + int64_t(k < nc ? k : k0) * kHeadDim);
+            }
+#pragma unroll
+          for (int h = 0; h < kOct; ++h) {
+            float a[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const float x0 = k01.x - c[h][q].x, x1 = k01.y - c[h][q].y, x2 = k23.x - c[h][q].z, x3 = k23.y - c[h][q].w;
+              a[q] = fmaf(x3, x3, fmaf(x2, x2, fmaf(x1, x1, x0 * x0)));
+            }
+            float bq[4], cq[2];
+#pragma unroll
+            for (int i2 = 0; i2 < 4; ++i2) {
+              const float send = b4 ? a[i2] : a[i2 + 4];
+              bq[i2] = (b4 ? a[i2 + 4] : a[i2]) + __shfl_xor_sync(0xffffffffu, send, 16);
+            }
+#pragma unroll
+            for (int i2 = 0; i2 < 2; ++i2) {
+              const float send = b3 ? bq[i2] : bq[i2 + 2];
+              cq[i2] = (b3 ? bq[i2 + 2] : bq[i2]) + __shfl_xor_sync(0xffffffffu, send, 8);
+            }
+            float dq = (b2 ? cq[1] : cq[0]) + __shfl_xor_sync(0xffffffffu, b2 ? cq[0] : cq[1], 4);
+            dq += __shfl_xor_sync(0xffffffffu, dq, 2);
+            dq += __shfl_xor_sync(0xffffffffu, dq, 1);
+            const int v = k0 + 8 * h + 4 * b4 + 2 * b3 + b2;
+            if ((lane & 3) == 0 && v < nc) dsm[t][v] = dq;
+          }
+        }
+        __syncthreads();
+        const int nc = mine ? min(kResChunk, r - kc) : 0;
+        // the fp32 best (distance, index)
+        for (int k = lane; k < nc; k += 32) {
+          const float d = dl[k];
+          const int j = kc + k;
+          if (d < bd || (d == bd && j < bj)) {
+            bd = d;
+            bj = j;
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float od = __shfl_xor_sync(0xffffffffu, bd, o);
+          const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+          if (od < bd || (od == bd && oj < bj)) {
+            bd = od;
+            bj = oj;
+          }
+        }
+        // the centres of the chunk whose interval reaches the best's so far
+        if (bj < r) hi = bd + bound(bd, bj);
+        for (int k0 = 0; k0 < nc; k0 += 32) {
+          const int k = k0 + lane;
+          bool m = false;
+          if (k < nc) {
+            const float d = dl[k];
+            m = !(d - bound(d, kc + k) > hi);
+          }
+          const unsigned bal = __ballot_sync(0xffffffffu, m);
+          if (na + __popc(bal) > kResChunk) over = true;
+          else if (m) jl[na + __popc(bal & ((1u << lane) - 1u))] = kc + k;
+          if (!over) na += __popc(bal);
+        }
+        __syncthreads();                                // dsm is refilled
       }
-      p.assign[int64_t(u) * p.s + pos] = res;
-      const int old = p.assign_prev ? p.assign_prev[int64_t(u) * p.s + pos] : -1;
-      if (res != old) {
-        atomicAdd(p.mcount + 2 * int64_t(u) * p.rmax + res, 1);
-        if (old >= 0) atomicAdd(p.mcount + (2 * int64_t(u) + 1) * p.rmax + min(old, r - 1), 1);
+      int res = bj;
+      if (mine && bj < r && (na > 1 || over)) {       // fp64 decides among them
+        float2 k01, k23;
+        key(tok, k01, k23);
+        const double kx[4] = {k01.x, k01.y, k23.x, k23.y};
+        const double* c64 = p.centers64 + int64_t(tok.x) * p.rmax * kHeadDim + 4 * lane;
+        double bd64 = INFINITY;
+        int bj64 = INT_MAX;
+        const int nq = over ? r : na;
+        for (int k0 = 0; k0 < nq; k0 += 4) {
+          int jq[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) jq[q] = k0 + q < nq ? (over ? k0 + q : jl[k0 + q]) : -1;
+          double a[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const double4_32a c =
+                *reinterpret_cast<const double4_32a*>(c64 + int64_t(jq[q] < 0 ? 0 : jq[q]) * kHeadDim);
+            double tt = (kx[0] - c.x) * (kx[0] - c.x);
+            tt = fma(kx[1] - c.y, kx[1] - c.y, tt);
+            tt = fma(kx[2] - c.z, kx[2] - c.z, tt);
+            a[q] = fma(kx[3] - c.w, kx[3] - c.w, tt);
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const double dd = __shfl_sync(0xffffffffu, a[q], 0);
+            if (jq[q] >= 0 && (dd < bd64 || (dd == bd64 && jq[q] < bj64))) {
+              bd64 = dd;
+              bj64 = jq[q];
+            }
+          }
+        }
+        res = bj64;
       }
+      if (mine && lane == 0) settle(tok.x, r, tok.y, res);
     }
-    __syncwarp();                                       // dl / jl are reused by the next token
+    __syncthreads();
+    if (threadIdx.x == 0) queued = 0;
+    __syncthreads();
   }
 }
 
