@@ -464,8 +464,10 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   const size_t sm_top = n_sort * 12;
   const size_t sm_scatter = size_t(std::max(rmax, 1)) * 4 * sizeof(int);
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
-      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false>, sm_scatter) != cudaSuccess ||
-      set_smem(k_lloyd_scatter<true>, sm_scatter) != cudaSuccess ||
+      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false, 1>, sm_scatter) != cudaSuccess ||
+      set_smem(k_lloyd_scatter<true, 1>, sm_scatter) != cudaSuccess ||
+      set_smem(k_lloyd_scatter<false, 4>, sm_scatter) != cudaSuccess ||
+      set_smem(k_lloyd_scatter<true, 4>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_assign<1>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<2>, kAsgSmemMax) != cudaSuccess ||
       set_smem(k_lloyd_assign<3>, kAsgSmemMax) != cudaSuccess ||
@@ -619,7 +621,9 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       // segments of at most 256 centres, of equal width
       const int nseg = int(cdiv(r_hi, kAsgRmax));
       const int segw = (int(cdiv(r_hi, nseg)) + 15) & ~15;
-      const dim3 gs(unsigned(cdiv(s, int64_t(kScatterThreads))), unsigned(U));
+      // tokens per thread of the list kernel: four where two CTAs per SM remain
+      const int tok = cdiv(s, int64_t(4 * kScatterThreads)) * U >= 2 * c->num_sms ? 4 : 1;
+      const dim3 gs(unsigned(cdiv(s, int64_t(tok * kScatterThreads))), unsigned(U));
       const dim3 ga(unsigned(cdiv(s, int64_t(kAccRows))), unsigned(U));
       auto clear = [&](int32_t* counts, size_t n) {
         return cudaMemsetAsync(counts, 0, n * sizeof(int32_t), stream) == cudaSuccess;
@@ -641,13 +645,15 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
           la.test_fault = 0;
         }
         k_lloyd_resolve<<<unsigned(3 * c->num_sms), kResWarps * 32, 0, stream>>>(la, int(asg_grid));
-        k_lloyd_scatter<false><<<gs, kScatterThreads, size_t(r_hi) * 4 * sizeof(int), stream>>>(la);
+        (tok == 4 ? k_lloyd_scatter<false, 4> : k_lloyd_scatter<false, 1>)
+            <<<gs, kScatterThreads, size_t(r_hi) * 4 * sizeof(int), stream>>>(la);
         (k16 ? k_lloyd_accum<false, true> : k_lloyd_accum<false, false>)<<<ga, kThreads, kAccSmem, stream>>>(la);
         if (last) {                       // the values of every member
           if (it > 0) {
             if (!clear(la.cursor, UR * rstride * 2))
               return fail(RESKV_ERR_CUDA, "clearing the list cursors");
-            k_lloyd_scatter<true><<<gs, kScatterThreads, size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
+            (tok == 4 ? k_lloyd_scatter<true, 4> : k_lloyd_scatter<true, 1>)
+                <<<gs, kScatterThreads, size_t(r_hi) * 2 * sizeof(int), stream>>>(la);
           }
           (v16 ? k_lloyd_accum<true, true> : k_lloyd_accum<true, false>)<<<ga, kThreads, kAccSmem, stream>>>(la);
         }

@@ -1145,14 +1145,17 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_init(LloydArgs p) {
 // sums are integers).  kMembers = false: the tokens whose centre changed in this
 // iteration, once by the centre they joined and once by the one they left (in the
 // first iteration every evicted token joins); kMembers = true: every member by
-// its centre.  A CTA takes 1024 tokens of a unit: it counts them per group in
-// shared memory, takes each group's place in its list with one atomic, and
+// its centre.  A CTA takes 1024 kTok tokens of a unit: it counts them per group
+// in shared memory, takes each group's place in its list with one atomic, and
 // writes the positions.  The groups start at the exclusive prefix of their
 // sizes, which every CTA of the unit forms again.  Dynamic shared memory: 4 r
 // ints.
+// What bounds it: the barriers and the prefix of every CTA, so a CTA takes 4096
+// tokens where that still leaves two CTAs per SM (64 units of 32K keys: 26 -> 21
+// us; 32 units of 128K: 47 -> 34; 512 of 16K: 75 -> 53), else 1024.
 constexpr int kScatterThreads = 1024;
 
-template <bool kMembers>
+template <bool kMembers, int kTok>
 __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) {
   extern __shared__ int sc_raw[];
   __shared__ int warp_sums[32];
@@ -1170,11 +1173,16 @@ __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) 
     else
       return (p.assign_prev ? p.ccount[c0 + g] : 0) + p.mcount[2 * c0 + g] - p.mcount[2 * c0 + p.rmax + g];
   };
-  const int64_t pos = int64_t(blockIdx.x) * kScatterThreads + threadIdx.x;
-  int a = -1, o = -1;                        // the token's centre now and before
-  if (pos < p.s) {
-    a = p.assign[int64_t(u) * p.s + pos];
-    if (!kMembers && p.assign_prev) o = p.assign_prev[int64_t(u) * p.s + pos];
+  const int64_t pos0 = int64_t(blockIdx.x) * kTok * kScatterThreads + threadIdx.x;
+  int a[kTok], o[kTok];                      // the tokens' centres now and before
+#pragma unroll
+  for (int t = 0; t < kTok; ++t) {
+    const int64_t pos = pos0 + t * kScatterThreads;
+    a[t] = o[t] = -1;
+    if (pos < p.s) {
+      a[t] = p.assign[int64_t(u) * p.s + pos];
+      if (!kMembers && p.assign_prev) o[t] = p.assign_prev[int64_t(u) * p.s + pos];
+    }
   }
   for (int g = threadIdx.x; g < ng; g += kScatterThreads) cnt[g] = 0;
   const int per = (ng + kScatterThreads - 1) / kScatterThreads, g0 = threadIdx.x * per;
@@ -1188,26 +1196,33 @@ __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) 
     if (blockIdx.x == 0) p.lbase[slot(g)] = base;
     base += size(g);
   }
-  if (a >= r || o >= r) {                    // only after a failed assignment
-    report_status(p.status, kStatusBadIndex);
-    a = o = -1;
+  int ra[kTok], ro[kTok];
+#pragma unroll
+  for (int t = 0; t < kTok; ++t) {
+    if (a[t] >= r || o[t] >= r) {            // only after a failed assignment
+      report_status(p.status, kStatusBadIndex);
+      a[t] = o[t] = -1;
+    }
+    if (!kMembers && a[t] == o[t]) a[t] = o[t] = -1;   // not moved
+    ra[t] = a[t] >= 0 ? atomicAdd(&cnt[a[t]], 1) : 0;
+    ro[t] = o[t] >= 0 ? atomicAdd(&cnt[r + o[t]], 1) : 0;
   }
-  if (!kMembers && a == o) a = o = -1;       // not moved
-  const int ra = a >= 0 ? atomicAdd(&cnt[a], 1) : 0;
-  const int ro = o >= 0 ? atomicAdd(&cnt[r + o], 1) : 0;
   __syncthreads();
   for (int g = threadIdx.x; g < ng; g += kScatterThreads)
     if (cnt[g] > 0) at[g] += atomicAdd(p.cursor + slot(g), cnt[g]);
   __syncthreads();
-  auto put = [&](int off) {
+  auto put = [&](int off, int t) {
     if (off < 0 || off >= 2 * p.s) {         // counts inconsistent with the assignment: the same
       report_status(p.status, kStatusBadIndex);
       return;
     }
-    p.list[2 * int64_t(u) * p.s + off] = int32_t(pos);
+    p.list[2 * int64_t(u) * p.s + off] = int32_t(pos0 + t * kScatterThreads);
   };
-  if (a >= 0) put(at[a] + ra);
-  if (o >= 0) put(at[r + o] + ro);
+#pragma unroll
+  for (int t = 0; t < kTok; ++t) {
+    if (a[t] >= 0) put(at[a[t]] + ra[t], t);
+    if (o[t] >= 0) put(at[r + o[t]] + ro[t], t);
+  }
 }
 
 // New centre = mean key of its members; on the last iteration also the mean
