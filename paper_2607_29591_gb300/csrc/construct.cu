@@ -715,7 +715,8 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
                 ent_stride, cfg.beta, int64_t(l) * UL, c->kslots, c->vslots, c->logc,
                 c->slot_pos, c->counts, c->n_main, c->n_res, bl_d,
                 per_unit ? c->offsets : nullptr};
-    k_pack<<<UL, 1024, 0, stream>>>(pa);
+    if (launch_clusters(k_pack, UL, c->num_sms, 0, stream, pa) != cudaSuccess)
+      return cleanup_fail(fail(RESKV_ERR_CUDA, "packing launch"));
     RESKV_LAUNCH_CHECK("packing");
     timing_ok &= timer.mark(-1);
     timing_ok &= timer.flush(c->build_ms);

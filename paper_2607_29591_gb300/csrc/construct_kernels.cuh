@@ -2130,9 +2130,19 @@ struct PackArgs {
   const int32_t* offsets;      // [U + 1] first slot of every unit, or NULL (u * stride)
 };
 
-__global__ void __launch_bounds__(1024) k_pack(PackArgs p) {
+// One cluster per unit, as for the ranking: its CTAs take equal runs of
+// positions, a warp 32 consecutive ones at a time, to list the main cache's in
+// ascending order, then all warps of the cluster copy the rows.  What bounds it:
+// the latency of few CTAs.  32 units of 128K keys, b = 2048: 27 us, 180 with one
+// CTA per unit and a run of positions per thread; 64 units of 32K keys: 26, 63;
+// 512 of 16K (one CTA each): 51, 59.
+__global__ void __launch_bounds__(kTopThreads) k_pack(PackArgs p) {
   __shared__ int warp_sums[32];
-  const int ul = blockIdx.x;
+  __shared__ int cta_total;
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = int(cl.num_blocks()), rank = int(cl.block_rank());
+  const int ul = blockIdx.x / cs;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t u = p.unit0 + ul;
   const int r = p.r_final[ul];
   const int64_t bu = unit_budget(p.budgets, ul, p.budget);
@@ -2141,26 +2151,48 @@ __global__ void __launch_bounds__(1024) k_pack(PackArgs p) {
   const int32_t* rp = p.rank_pos + int64_t(ul) * p.s;
   const int64_t base = p.offsets ? int64_t(p.offsets[u]) : u * p.stride;   // first slot of u
   int32_t* spos = p.slot_pos + base;
-  const int64_t chunk = (p.s + blockDim.x - 1) / blockDim.x;
-  const int64_t lo = int64_t(threadIdx.x) * chunk, hi = lo + chunk < p.s ? lo + chunk : p.s;
+  // the warp's run of positions, a multiple of 32
+  const int64_t run = (p.s + int64_t(cs) * kTopThreads - 1) / (int64_t(cs) * kTopThreads) * 32;
+  const int64_t lo = (int64_t(rank) * (kTopThreads / 32) + w) * run, hi = lo + run < p.s ? lo + run : p.s;
+  const int steps = lo < hi ? int((hi - lo + 31) >> 5) : 0;
+  auto main_pos = [&](int64_t i, int32_t rk) { return i < hi && (rk < 0 || rk < keep); };
+  unsigned saved = 0;                            // lane k: the bits of step k (of the first 32)
   int mine = 0;
-  for (int64_t i = lo; i < hi; ++i) {
-    const int32_t rk = rp[i];
-    mine += (rk < 0 || rk < keep);
-  }
-  int out = block_exclusive_scan(mine, warp_sums, nullptr);
-  for (int64_t i = lo; i < hi; ++i) {
-    const int32_t rk = rp[i];
-    if (rk < 0 || rk < keep) {
-      if (out < m) spos[out] = int32_t(i);
-      ++out;
+  for (int k0 = 0; k0 < steps; k0 += 8) {        // eight loads in flight
+    int32_t rk[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int64_t i = lo + 32 * int64_t(k0 + k) + lane;
+      rk[k] = i < hi ? __ldg(rp + i) : INT_MAX;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const unsigned f = __ballot_sync(0xffffffffu, main_pos(lo + 32 * int64_t(k0 + k) + lane, rk[k]));
+      if (lane == k0 + k) saved = f;
+      mine += __popc(f);
     }
   }
+  if (lane == 0) warp_sums[w] = mine;
   __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int out = 0;                                   // main positions before the warp's
+  for (int k = 0; k < w; ++k) out += warp_sums[k];
+  if (threadIdx.x == kTopThreads - 1) cta_total = out + mine;
+  cl.sync();
+  for (int k = 0; k < rank; ++k) out += *cl.map_shared_rank(&cta_total, k);
+  for (int k = 0; k < steps; ++k) {
+    const int64_t i = lo + 32 * int64_t(k);
+    const unsigned f = k < 32 ? __shfl_sync(0xffffffffu, saved, k)
+                              : __ballot_sync(0xffffffffu, main_pos(i + lane, i + lane < hi ? rp[i + lane] : INT_MAX));
+    const int at = out + __popc(f & ((1u << lane) - 1u));
+    if ((f >> lane & 1u) && at < m) spos[at] = int32_t(i + lane);
+    out += __popc(f);
+  }
+  cl.sync();                                     // the list is complete (and cta_total read)
+  const int w0 = rank * (kTopThreads / 32) + w, nw = cs * (kTopThreads / 32);
   const __nv_bfloat16* Ku = p.K + int64_t(ul) * p.s * kHeadDim;
   const __nv_bfloat16* Vu = p.V + int64_t(ul) * p.s * kHeadDim;
-  for (int64_t j = w; j < m; j += nw) {
+#pragma unroll 2
+  for (int64_t j = w0; j < m; j += nw) {
     const int64_t pos = spos[j];
     const uint2 kw = __ldg(reinterpret_cast<const uint2*>(Ku + pos * kHeadDim) + lane);
     const uint2 vw = __ldg(reinterpret_cast<const uint2*>(Vu + pos * kHeadDim) + lane);
@@ -2172,7 +2204,7 @@ __global__ void __launch_bounds__(1024) k_pack(PackArgs p) {
     }
   }
   const int c = p.chosen[ul];
-  for (int j = w; j < r; j += nw) {
+  for (int j = w0; j < r; j += nw) {
     const int64_t e = int64_t(ul) * p.ent_stride + p.run_off[c] + j;
     const int64_t slot = base + m + j;
     reinterpret_cast<uint2*>(p.kslots + slot * kHeadDim)[lane] =
@@ -2186,7 +2218,7 @@ __global__ void __launch_bounds__(1024) k_pack(PackArgs p) {
       spos[m + j] = -1;
     }
   }
-  if (threadIdx.x == 0) {
+  if (rank == 0 && threadIdx.x == 0) {
     p.n_main[u] = int32_t(m);
     p.n_res[u] = r;
   }
