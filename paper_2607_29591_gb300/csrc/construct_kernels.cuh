@@ -952,7 +952,7 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_topk(TopArgs p) {
 // (score desc, head asc, position asc).  One cluster per batch element: a radix
 // select of the n_free-th largest key over the heads' remaining tokens, then
 // per-head counts above and at the threshold.  (One CTA and eight 8-bit digits
-// took 1043 us for 8 heads of 32K tokens, this 99.)
+// took 1043 us for 8 heads of 32K tokens, this with one load at a time 98, now 70.)
 // ---------------------------------------------------------------------------
 
 struct AdaArgs {
@@ -985,11 +985,23 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_adakv(AdaArgs p) {
   for (int h = rank * kTopThreads + threadIdx.x; h < 2 * H; h += cs * kTopThreads) p.counts[2 * ul0 + h] = 0;
   // f(head, key) for the remaining tokens of this CTA's positions of every head
   const int64_t lo = n_ev * rank / cs, hi = n_ev * (rank + 1) / cs;
+  // (eight loads in flight; not the head's safeguard tokens)
   auto each = [&](int h, auto&& f) {
     const double* sc = p.scores + int64_t(ul0 + h) * s;
     const int32_t* rp = p.rank_pos + int64_t(ul0 + h) * s;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += kTopThreads)
-      if (rp[i] >= p.f) f(score_key(sc[i]));    // not the head's safeguard token
+    for (int64_t i = lo + threadIdx.x; i < hi; i += 8 * kTopThreads) {
+      double v[8];
+      bool take[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int64_t x = i + j * kTopThreads;
+        v[j] = x < hi ? __ldg(sc + x) : 0.0;
+        take[j] = x < hi && __ldg(rp + x) >= p.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (take[j]) f(score_key(v[j]));
+    }
   };
   const SelState st = cluster_select(cl, p.n_free, hist, warp_sums, bcast, [&](auto&& f) {
     for (int h = 0; h < H; ++h) each(h, f);
@@ -1478,10 +1490,24 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * kFinWarps + (threadIdx.x >> 5), u = blockIdx.y, ul = u % p.UL;
   const int r = p.r_unit[u];
+  // members of the block's centres and their rounded reciprocals: one fp64
+  // division for all of them
+  __shared__ int cnt_s[kFinWarps];
+  __shared__ double rcp_s[kFinWarps];
+  if (threadIdx.x < kFinWarps) {
+    const int jj = blockIdx.x * kFinWarps + threadIdx.x;
+    int n = 0;
+    if (jj < r) {
+      const int32_t* mc = p.mcount + 2 * int64_t(u) * p.rmax + jj;
+      n = (p.assign_prev ? p.ccount[int64_t(u) * p.rmax + jj] : 0) + mc[0] - mc[p.rmax];
+    }
+    cnt_s[threadIdx.x] = n;
+    rcp_s[threadIdx.x] = n > 0 ? (1.0 / double(n)) * 0x1p-32 : 0.0;
+  }
+  __syncthreads();
   if (j >= r) return;
   const int64_t uj = int64_t(u) * p.rmax + j;
-  const int32_t* mc = p.mcount + 2 * int64_t(u) * p.rmax + j;
-  const int cnt = (p.assign_prev ? p.ccount[uj] : 0) + mc[0] - mc[p.rmax];
+  const int cnt = cnt_s[threadIdx.x >> 5];
   const uint32_t flag = p.mflag[uj];
   const bool exact = flag == 0u;
   // dim 4 lane + q of the key sums at 32 q, of the value sums at kHeadDim + 32 q
@@ -1495,7 +1521,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   double tk[4], tv[4], mk[4], mv[4];
   const double cd = double(cnt);
   if (exact) {
-    const double y = cnt > 0 ? (1.0 / cd) * 0x1p-32 : 0.0;
+    const double y = rcp_s[threadIdx.x >> 5];
     const double bd = cd * 0x1p32;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -1592,7 +1618,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     }
     if (lane == 0) p.ecount[e] = cnt;
   }
-  __syncwarp();                       // every lane has read mflag and ccount
+  __syncwarp();                       // every lane has read mflag
   if (lane == 0) {
     p.cnorm[uj] = n;
     p.ccount[uj] = cnt;
