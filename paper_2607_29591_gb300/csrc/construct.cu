@@ -498,7 +498,8 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       k_obs_pass1<<<dim3(ntiles, UL), 32 * obs_warps1(n_fit_rows), sm_obs1, stream>>>(oa);
       k_obs_rowstats<<<unsigned(cdiv(int64_t(UL) * n_fit_rows, 32)), 256, 0, stream>>>(oa, UL);
       k_obs_pass2<<<dim3(ntiles, UL), 32 * obs_warps2(n_fit_rows), sm_obs2, stream>>>(oa);
-      k_pool<<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(A, scores, s, UL, cfg.pool_kernel);
+      k_pool<<<unsigned(cdiv(int64_t(UL) * cdiv(s, int64_t(4)), 256)), 256, 0, stream>>>(A, scores, s, UL, cfg.pool_kernel,
+                                                                                     1.0 / double(cfg.pool_kernel));
     } else {
       k_key_norms<true><<<unsigned(cdiv(int64_t(US), 256)), 256, 0, stream>>>(K, scores, knorm, int64_t(US));
     }

@@ -379,18 +379,35 @@ __global__ void __launch_bounds__(128, 3) k_obs_pass2(ObsArgs p) {
   }
 }
 
-// Zero-padded average pooling of width `pool` (odd), summed in fp64.
-__global__ void k_pool(const float* A, double* scores, int64_t s, int UL, int pool) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= int64_t(UL) * s) return;
-  const int64_t ul = i / s, pidx = i % s;
+// Zero-padded average pooling of width `pool` (odd), summed in fp64 in ascending
+// order; inv = RN(1 / pool).  Bound by fp64, scarce on this part: a thread takes
+// four positions, so a value is converted once for them, and divides by
+// Markstein's correction (q0 = RN(a inv), r = a - q0 pool exactly, q = RN(q0 + r inv):
+// with an odd divisor a / pool lies at least 1 / (2 pool) ulp from a rounding
+// boundary, far more than the correction is off by).  4.2M positions, width 7: 107
+// us, 150 with a conversion per term and a division.
+__global__ void __launch_bounds__(256) k_pool(const float* __restrict__ A, double* __restrict__ scores, int64_t s, int UL,
+                                              int pool, double inv) {
+  const int64_t runs = (s + 3) / 4, i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= int64_t(UL) * runs) return;
+  const int64_t ul = i / runs, p0 = i % runs * 4;
+  const float* Au = A + ul * s;
   const int half = pool / 2;
-  double acc = 0.0;
-  for (int j = -half; j <= half; ++j) {
-    const int64_t q = pidx + j;
-    if (q >= 0 && q < s) acc += double(A[ul * s + q]);
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int j = -half; j < half + 4; ++j) {       // value p0 + j belongs to positions p0 + j - half .. p0 + j + half
+    const int64_t q = p0 + j;
+    if (q < 0 || q >= s) continue;
+    const double v = double(__ldg(Au + q));
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (j >= k - half && j <= k + half) acc[k] += v;
   }
-  scores[i] = acc / double(pool);
+  const double n = double(pool);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double q0 = acc[k] * inv;
+    if (p0 + k < s) scores[ul * s + p0 + k] = fma(fma(-q0, n, acc[k]), inv, q0);
+  }
 }
 
 // Query-free score ||k_p||^2 (a build choice; the paper defines none): the
