@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(256) k_pool(const float* __restrict__ A, doubl
 // (k_key_norms): every nonzero value lies within 20 binades of the largest, so
 // all values are integers below 2^28 in units of the lowest of those binades,
 // their squares sum below 2^63 in 64-bit integers, one multiply-add each, and
-// one conversion rounds the sum.  Otherwise a warp takes the row
+// one conversion rounds the sum (within 13 binades a float addition forms the
+// integer, else a shift).  Otherwise a warp takes the row
 // (keynorm_row): with tmax the largest t of the row's nonzero squares, every
 // square with t >= tmax - 104 is an exact integer multiple of 2^(tmax - 104)
 // below 2^120, and 128 of them sum below 2^127: it adds them as 128-bit
@@ -549,7 +550,8 @@ __device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.
 // loads), and every lane keeps the sum of one row,
 // so the conversion and the root are done once for 32 rows.  Memory bound in
 // principle (256 bytes a row); the integer sums issue about as long as the
-// loads take.  8.4M rows: 642 us for score and bound together, 2883 + 768 with a
+// loads take.  8.4M rows: 505 us for score and bound together (645 with shifts
+// for every row), 2883 + 768 with a
 // warp per row and 128-bit sums; the bound alone, 2.1M rows: 77 us, 194.
 template <bool kScore>
 __global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restrict__ K, double* __restrict__ scores,
@@ -599,19 +601,37 @@ __global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restri
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) mm = max_s16x2(mm, __shfl_xor_sync(0xffffffffu, mm, o));
         const int emax = int(mm & 0xffffu) >> 7, umin = 0x8000 - (int(mm) >> 16);
-        const int elow = emax - 20;
+        // 13 binades (four rows of normally distributed values nearly always):
+        // a float addition of 1.5 x 2^23 units leaves M in the low bits
+        const bool near = emax >= 14 && emax <= 251 && umin >= ((emax - 13) << 7);
+        const bool all_near = __all_sync(0xffffffffu, near);
+        const int elow = all_near ? emax - 13 : emax - 20;
         uint64_t s64 = 0;
+        if (all_near) {
+          const uint32_t cb = (uint32_t(elow + 16) << 23) | 0x400000u;
+          const float2 c2 = make_float2(__uint_as_float(cb), __uint_as_float(cb));
+          long long acc = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-          for (int hw = 0; hw < 2; ++hw) {
-            const uint32_t u = hw ? x[j] >> 16 : x[j];
-            const int e = int((u >> 7) & 0xffu);
-            // 2^(e - elow) M: zero (all bits shifted out) below elow
-            uint32_t m;
-            asm("shl.b32 %0, %1, %2;" : "=r"(m) : "r"((u & 0x7fu) | 0x80u), "r"(e - elow));
-            s64 += uint64_t(m) * m;
+          for (int j = 0; j < 8; ++j) {
+            const float2 y = fadd2(bf16x2_to_float2(x[j]), c2);
+            const int m0 = int(__float_as_uint(y.x) - cb), m1 = int(__float_as_uint(y.y) - cb);
+            acc += (long long)m0 * m0;
+            acc += (long long)m1 * m1;
           }
+          s64 = uint64_t(acc);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int hw = 0; hw < 2; ++hw) {
+              const uint32_t u = hw ? x[j] >> 16 : x[j];
+              const int e = int((u >> 7) & 0xffu);
+              // 2^(e - elow) M: zero (all bits shifted out) below elow
+              uint32_t m;
+              asm("shl.b32 %0, %1, %2;" : "=r"(m) : "r"((u & 0x7fu) | 0x80u), "r"(e - elow));
+              s64 += uint64_t(m) * m;
+            }
+        }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) s64 += __shfl_xor_sync(0xffffffffu, s64, o);
         if (c == 4 * half + i) {

@@ -57,3 +57,29 @@ def test_scores(s, r):
     Kd = K[0, 0].double().numpy()
     ref = np.array([math.inf if np.isinf(x).any() else math.fsum(x * x) for x in Kd])
     assert np.array_equal(got, ref), np.nonzero(got != ref)[0][:5]
+
+
+@pytest.mark.parametrize("span", [11, 12, 13, 14])
+@pytest.mark.parametrize("top", [-120, -112, -111, 0, 123, 124, 125])
+def test_scores_of_narrow_rows(span, top):
+    """Every row spans `span` binades (13 is the last that float additions take),
+    at the largest exponents on both sides of that form's range; one row in 40
+    spans more, so that its neighbours leave the form too."""
+    s = 164
+    g = torch.Generator().manual_seed(span)
+    e = torch.randint(-span, 1, (s, 128), generator=g)
+    K = (1 + torch.randint(0, 128, (s, 128), generator=g) / 128) * torch.exp2(e.float()) * 2.0 ** top
+    K[:, 3], K[:, 77] = 1.9921875 * 2.0 ** top, 1.0078125 * 2.0 ** max(top - span, -126)
+    K[::40, 5] = 2.0 ** max(top - 18, -133)
+    K[:, 1::2] *= -1
+    K[:, 9] = 0
+    K = K.to(torch.bfloat16)[None, None]
+    cfg = R.reskv_config_default(batch=1, n_layers=1, n_kv_heads=1, group=4, seq_len=s, budget=80, n_obs=0, n_fit=0,
+                                 n_val=0, score_mode=R.RESKV_SCORE_KEYNORM,
+                                 residual_override=np.zeros(1, np.int32), keep_debug=1)
+    cache = R.reskv_build_cache(cfg, [K.cuda()], [K.cuda()], None)
+    R.reskv_check_status(cache)
+    got = R.reskv_export_debug(cache, R.RESKV_DEBUG_SCORES).ravel()
+    cache.free()
+    ref = np.array([math.fsum(x * x) for x in K[0, 0].double().numpy()])
+    assert np.array_equal(got, ref), np.nonzero(got != ref)[0][:5]
