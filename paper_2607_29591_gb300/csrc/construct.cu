@@ -463,8 +463,9 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   while (n_sort < size_t(std::max(n_top, 1))) n_sort *= 2;
   const size_t sm_top = n_sort * 12;
   const size_t sm_scatter = size_t(std::max(rmax, 1)) * 4 * sizeof(int);
+  auto* topk_k = n_top <= 2 * kTopThreads ? k_topk<2> : k_topk<8>;
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
-      set_smem(k_topk, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false, 1>, sm_scatter) != cudaSuccess ||
+      set_smem(k_topk<2>, sm_top) != cudaSuccess || set_smem(k_topk<8>, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false, 1>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_scatter<true, 1>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_scatter<false, 4>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_scatter<true, 4>, sm_scatter) != cudaSuccess ||
@@ -510,7 +511,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
     if (adakv) {
       // AdaKV: mark every head's safeguard (its top f), split the shared slots
       TopArgs tf{scores, s, P, ada_f, top, rank_pos, c->status, nullptr};
-      const cudaError_t e1 = launch_clusters(k_topk, UL, c->num_sms, sm_top, stream, tf);
+      const cudaError_t e1 = launch_clusters(topk_k, UL, c->num_sms, sm_top, stream, tf);
       AdaArgs aa{scores, rank_pos, s, P, cfg.n_kv_heads, ada_f, P + ada_f,
                  int64_t(cfg.n_kv_heads) * (n_free_head - ada_f), bl_d, ada_counts};
       const cudaError_t e2 = launch_clusters(k_adakv, cfg.batch, c->num_sms, 0, stream, aa);
@@ -545,7 +546,7 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
         cudaMemsetAsync(top, 0xff, size_t(UL) * n_top * 4, stream) != cudaSuccess)
       return cleanup_fail(fail(RESKV_ERR_CUDA, "clearing the ranking"));
     TopArgs ta{scores, s, P, n_top, top, rank_pos, c->status, bl_d};
-    if (launch_clusters(k_topk, UL, c->num_sms, sm_top, stream, ta) != cudaSuccess)
+    if (launch_clusters(topk_k, UL, c->num_sms, sm_top, stream, ta) != cudaSuccess)
       return cleanup_fail(fail(RESKV_ERR_CUDA, "launching the ranking"));
     RESKV_LAUNCH_CHECK("ranking");
     // candidate r per unit of this layer

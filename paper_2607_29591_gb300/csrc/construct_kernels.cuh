@@ -889,8 +889,12 @@ __device__ void topk_rank(const TopArgs& p, int ul, int K, uint64_t* skey, int32
   }
 }
 
-// Launched in clusters of 1 to 8 CTAs per unit.
-__global__ void __launch_bounds__(kTopThreads, 1) k_topk(TopArgs p) {
+// Launched in clusters of 1 to 8 CTAs per unit; n_top at most kMaxE kTopThreads.
+// (Where a unit has one CTA, two of them per SM cover each other's barriers: 32
+// registers, which the sort of 4 or 8 keys per thread does not fit.  512 units of
+// 16K keys, n_top = 64: 160 us -> 136.)
+template <int kMaxE>
+__global__ void __launch_bounds__(kTopThreads, kMaxE <= 2 ? 2 : 1) k_topk(TopArgs p) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) uint8_t smraw[];
   int n_sort = kTopThreads;                      // the power of two that holds n_top
@@ -974,10 +978,16 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_topk(TopArgs p) {
   }
   cl.sync();                                   // the list is complete; nobody reads another CTA's memory after
   if (rank != 0) return;
-  if (K <= kTopThreads) topk_rank<1>(p, ul, K, skey, sidx);
-  else if (K <= 2 * kTopThreads) topk_rank<2>(p, ul, K, skey, sidx);
-  else if (K <= 4 * kTopThreads) topk_rank<4>(p, ul, K, skey, sidx);
-  else topk_rank<8>(p, ul, K, skey, sidx);
+  if (K <= kTopThreads) {
+    topk_rank<1>(p, ul, K, skey, sidx);
+  } else if (kMaxE == 2 || K <= 2 * kTopThreads) {
+    topk_rank<2>(p, ul, K, skey, sidx);
+  } else {
+    if constexpr (kMaxE > 2) {
+      if (K <= 4 * kTopThreads) topk_rank<4>(p, ul, K, skey, sidx);
+      else topk_rank<8>(p, ul, K, skey, sidx);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
