@@ -547,12 +547,11 @@ __device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.
 //
 // A warp takes 32 rows, four at a time with eight lanes each (two 16-byte loads
 // a lane, four rows' worth in flight; keys on an 8-byte boundary take 8-byte
-// loads), and every lane keeps the sum of one row,
-// so the conversion and the root are done once for 32 rows.  Memory bound in
-// principle (256 bytes a row); the integer sums issue about as long as the
-// loads take.  8.4M rows: 505 us for score and bound together (645 with shifts
-// for every row), 2883 + 768 with a
-// warp per row and 128-bit sums; the bound alone, 2.1M rows: 77 us, 194.
+// loads), and every lane keeps the sum of one row, so the conversion and the root
+// are done once for 32 rows.  The bound alone runs at the DRAM rate (2.1M rows: 77
+// us, 194 with a warp per row); with the scores the integer sums issue for longer
+// than the loads take (8.4M rows, 2.1 GB: 505 us for both, 645 with shifts for
+// every row, 2883 + 768 with a warp per row and 128-bit sums).
 template <bool kScore>
 __global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restrict__ K, double* __restrict__ scores,
                                                    float* __restrict__ knorm, int64_t n_rows) {
