@@ -463,7 +463,9 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   while (n_sort < size_t(std::max(n_top, 1))) n_sort *= 2;
   const size_t sm_top = n_sort * 12;
   const size_t sm_scatter = size_t(std::max(rmax, 1)) * 4 * sizeof(int);
-  auto* topk_k = n_top <= 2 * kTopThreads ? k_topk<2> : k_topk<8>;
+  // two ranking CTAs per SM where there are more units than SMs (else one has an SM
+  // to itself, and 32 registers only spill: 32 units of 128K 93 -> 97 us)
+  auto* topk_k = UL > c->num_sms && n_top <= 2 * kTopThreads ? k_topk<2> : k_topk<8>;
   if (set_smem(k_obs_pass1, sm_obs1) != cudaSuccess || set_smem(k_obs_pass2, sm_obs2) != cudaSuccess ||
       set_smem(k_topk<2>, sm_top) != cudaSuccess || set_smem(k_topk<8>, sm_top) != cudaSuccess || set_smem(k_lloyd_scatter<false, 1>, sm_scatter) != cudaSuccess ||
       set_smem(k_lloyd_scatter<true, 1>, sm_scatter) != cudaSuccess ||

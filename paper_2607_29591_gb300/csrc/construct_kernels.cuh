@@ -889,7 +889,7 @@ __device__ void topk_rank(const TopArgs& p, int ul, int K, uint64_t* skey, int32
 }
 
 // Launched in clusters of 1 to 8 CTAs per unit; n_top at most kMaxE kTopThreads.
-// (Where a unit has one CTA, two of them per SM cover each other's barriers: 32
+// (Where there are more units than SMs, two CTAs per SM cover each other's barriers: 32
 // registers, which the sort of 4 or 8 keys per thread does not fit.  512 units of
 // 16K keys, n_top = 64: 160 us -> 136.)
 template <int kMaxE>
