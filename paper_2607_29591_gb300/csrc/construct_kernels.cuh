@@ -1134,7 +1134,7 @@ struct LloydArgs {
                                // those that left, grouped by centre (or every member, by centre)
   long long* msum;             // [U, rmax, 2, d] fixed-point member sums (K, V), dim 4 l + q at
                                // 32 q + l; zero between runs
-  long long* tsum;             // [U, rmax, 2, d] what the fixed-point sums dropped, unit 2^-76
+  long long* tsum;             // [U, rmax, 2, d] what the fixed-point sums dropped, unit 2^-kTailBits
   uint32_t* mflag;             // [U, rmax] kSumTails: tsum holds a part of the sum; kSumFp64: a
                                // member value is outside both
   __nv_bfloat16* kbar;         // [UL, ent_stride, d] entries, candidate c's at run_off[c]
@@ -1309,15 +1309,18 @@ __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) 
 // additions and a maximum per value.
 // A value is dropped from when it is below 2^-20 in magnitude (about 8 in
 // 10^7 of normally distributed values, so in a few of a unit's centres): the
-// warp then adds the exact e as 64-bit integers of unit 2^-76, kept beside and
-// flushed into tsum.  Sums that leave the binade (64 rows that sum past 4096) or
-// values with bits below 2^-76 flag the centre: it is summed in fp64 in member
-// order.
+// warp then adds the exact e as 64-bit integers of unit 2^-60, kept beside and
+// flushed into tsum.  |e| is at most half of T's grid, 2^32 units, so the 2^30
+// members that a centre can have sum to 2^62 at most.  Sums that leave the binade
+// (64 rows that sum past 4096) or values with bits below 2^-60 flag the centre: it
+// is summed in fp64 in member order.
 constexpr int kAccRowsPerWarp = 64;
 constexpr int kAccRows = kAccRowsPerWarp * (kThreads / 32);   // member slots per CTA
 constexpr float kSumC1 = 12288.0f;
 constexpr float kSumC2 = 0x1.8p-4f;
 static_assert(kAccRowsPerWarp <= 64, "T must stay within 2^-5 of C2");
+constexpr int kTailBits = 60;                                 // unit of a dropped part: 2^-60
+constexpr float kTailScale = 0x1p60f;
 enum : uint32_t { kSumFp64 = 1u, kSumTails = 2u };            // mflag
 
 struct PairSum {
@@ -1343,9 +1346,9 @@ __device__ __forceinline__ long long sum_total(float s, float t) {
   return (__float2ll_rz(s * 0x1p32f) - c1) + (__float2ll_rz(t * 0x1p32f) - c2);
 }
 
-// A dropped e as an integer of unit 2^-76; exact unless it has bits below.
+// A dropped e as an integer of unit 2^-kTailBits; exact unless it has bits below.
 __device__ __forceinline__ long long tail_units(float e, bool& ok) {
-  const float x = e * 0x1p76f;
+  const float x = e * kTailScale;
   const long long v = __float2ll_rz(x);
   ok &= fabsf(x) < 0x1p62f && __ll2float_rz(v) == x;
   return v;
@@ -1354,9 +1357,9 @@ __device__ __forceinline__ long long tail_units(float e, bool& ok) {
 // The lane's sums of four consecutive bf16 dims (two words, low half first).
 struct RowSum {
   PairSum a, b;
-  long long tail[4];             // the dropped parts, unit 2^-76
+  long long tail[4];             // the dropped parts, unit 2^-kTailBits
   uint32_t left;                 // OR of bits(S) ^ bits(C1)
-  bool dropped, bad;             // some lane's e was not zero; an e has bits below 2^-76
+  bool dropped, bad;             // some lane's e was not zero; an e has bits below its unit
 
   __device__ __forceinline__ void reset() {
     a = b = pair_zero();
@@ -1582,10 +1585,10 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
       }
     }
   } else if ((flag & kSumFp64) == 0u) {
-    // some values have bits below T's grid: sum = RN(S * 2^-32 + tails * 2^-76)
+    // some values have bits below T's grid: sum = RN(S * 2^-32 + tails * 2^-kTailBits)
     auto total = [](long long hi, long long lo) {
-      const __int128 v = (__int128(hi) << 44) + lo;
-      const double x = v == 0 ? 0.0 : round_u128(u128(v < 0 ? -v : v), -76, false);
+      const __int128 v = (__int128(hi) << (kTailBits - 32)) + lo;
+      const double x = v == 0 ? 0.0 : round_u128(u128(v < 0 ? -v : v), -kTailBits, false);
       return v < 0 ? -x : x;
     };
 #pragma unroll
