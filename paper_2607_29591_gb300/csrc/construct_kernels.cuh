@@ -538,8 +538,10 @@ __device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
 }
 
 // 128 fp32 products summed in any order stay within 130 u of the sum, the root
-// and the product within 2 u each
-__device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.0f + 140.0f * 5.9604645e-8f); }
+// and the product within 2 u each; what underflows is below 255 * 2^-150, its root
+// below kNormLost
+constexpr float kNormLost = 0x1p-70f;
+__device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.0f + 140.0f * 5.9604645e-8f) + kNormLost; }
 
 // Per key row, in one read of the keys: with kScore the query-free score, and
 // (knorm not NULL) an upper bound of ||k|| for the Lloyd assignment's rounding

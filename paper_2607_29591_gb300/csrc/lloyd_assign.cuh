@@ -63,6 +63,10 @@
 // 24 bits; 16 chained steps (both planes) give 272 * 2^-22 P = 1088u P, the split
 // e adds 256u P, |c1| + |c2| exceeds |c| by 2^-8: 1350u P, taken as 1440u P.  (A
 // bound three times as wide cost k_lloyd_resolve 1.7 to 2.1 times its time.)
+// Values, products and sums below 2^-126 may be lost besides, whole at worst: 2^-126
+// sum_i (|c_i| + |k_i|) <= 12 * 2^-126 (||c|| + ||k||) for the operands, twice that in a
+// distance, and some 600 terms of 2^-126.  So W is positive however small the
+// distances are, and centres at equal ones (all of them zero, say) are candidates.
 //
 // What bounds it: issue and the latency of a tile's steps (about 2.3 instructions
 // per cycle; the tensor pipe is active 28 % of the time at r = 51 and 54 % at 204,
@@ -408,11 +412,11 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
       const float d0 = fminf(min3(a[0], a[1], a[2]), a[3]);
       // A computed distance is off by at most ee + 4u |d| from the exact distance
       // to the fp64 centre: ee = 2 x dot product (gam_tc ||c|| ||k||, and 2u for
-      // the fp32 centre) + norm sum gam ||c||^2 (130u, and 2u for the fp32 centre),
-      // ||c|| <= max ||c|| over the unit.  So the nearest centre's computed
-      // distance is within 2 ee + 4u (|d0| + |d|) of d0.
+      // the fp32 centre) + norm sum gam ||c||^2 (130u, and 2u for the fp32 centre)
+      // + what underflows, ||c|| <= max ||c|| over the unit.  So the nearest
+      // centre's computed distance is within 2 ee + 4u (|d0| + |d|) of d0.
       const float uu = 5.9604645e-8f, gam = 140.0f * uu, gam_tc = 1440.0f * uu;
-      const float ee = cm * (2.0f * gam_tc * kn + gam * cm);
+      const float ee = fmaf(cm, 2.0f * gam_tc * kn + gam * cm, fmaf(0x1p-121f, kn + cm, 0x1p-116f));
       const float ww = 2.01f * ee;
       const float thr = d0 + asg_window(ww, d0);
       const float2 nthr = make_float2(-thr, -thr);
@@ -542,7 +546,7 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
           for (int i = lane; i < cm.r; i += 32) cmx = fmaxf(cmx, p.cnorm[c0 + i]);
   #pragma unroll
           for (int o = 16; o > 0; o >>= 1) cmx = fmaxf(cmx, __shfl_xor_sync(0xffffffffu, cmx, o));
-          cmx = sqrtf(cmx);
+          cmx = sqrtf(cmx) + kNormLost;
           const bool w = asg_wait(&sh.planes_full, uint32_t((nu - 1) & 1), &sh.abort);
           if (__any_sync(0xffffffffu, !w)) {
             ok = false;
@@ -702,7 +706,8 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
 // 16 u d32_j + 3 u ||c_j|| (sqrt(d32_j) + u ||c_j||) bounds the difference to
 // the exact distance D_j to the fp64 centre (12 u for the rounded differences,
 // the 4-term chain and the 5 butterfly levels; 2 u ||c|| (2 sqrt(D) + u ||c||)
-// for |c32 - c64| <= u ||c||; the rest is slack for using d32 in place of D).
+// for |c32 - c64| <= u ||c||; the rest is slack for using d32 in place of D); 2^-126
+// is added, far more than squares that underflow can lose.
 // The fp32 best decides unless another candidate's interval
 // [d32_j - b_j, d32_j + b_j] reaches the best's; those few are re-evaluated in
 // fp64, ties to the lower index.  Writes assign and counts the move.
@@ -755,7 +760,7 @@ __global__ void __launch_bounds__(kResWarps * 32, 3) k_lloyd_resolve(LloydArgs p
   };
   auto interval = [&](float d, float norm2) {
     const float cn = sqrtf(norm2) * 1.001f;
-    return 16.0f * uu * d + 3.0f * uu * cn * (sqrtf(d) + uu * cn);
+    return 16.0f * uu * d + 3.0f * uu * cn * (sqrtf(d) + uu * cn) + FLT_MIN;
   };
   // (four tokens nw apart: where there are few, every warp has one at most)
   for (int64_t i0 = 0; i0 < n; i0 += 4 * nw) {
