@@ -434,7 +434,10 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
         const uint32_t v = (((w[0] << 4) | w[1]) << 8) | (w[2] << 4) | w[3];
         m[i >> 1] |= (i & 1) ? v : v << 16;
       }
-      AsgCand cd{d0, 0, 0, min(__popc(m[0]) + __popc(m[1]), 3)};
+      // Below a window of 1e32 every product, sum and norm is finite.  Past it a
+      // centre may lie beside the token at a distance that overflowed, so all
+      // centres are candidates (where any distance is a number at all).
+      AsgCand cd{d0, 0, 0, ww < 1e32f ? min(__popc(m[0]) + __popc(m[1]), 3) : d0 < INFINITY ? 3 : 0};
       if (cd.n == 0) {                                    // no centre, or NaN or infinite distances
         cd.d = INFINITY;
       } else {
