@@ -229,6 +229,7 @@ __device__ int nearest_entry(const uint16_t* k, const uint16_t* kb, int nr) {
   const float2 k01 = bf16x2_to_float2(kw.x), k23 = bf16x2_to_float2(kw.y);
   const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1;
   if (threadIdx.x == 0) ncand = odd = 0;
+  __syncthreads();                      // (any warp may raise odd)
   float hi = INFINITY;                  // least upper end of an interval so far
   for (int c0 = 0; c0 < nr; c0 += kAppChunk) {
     const int nc = min(kAppChunk, nr - c0);
