@@ -1168,6 +1168,7 @@ __device__ __forceinline__ void split_planes(const LloydArgs& p, int u, int j, i
 }
 
 constexpr int kFinWarps = 8;
+constexpr int kFinScan = 8, kFinRows = 4;   // where a centre is summed in fp64: loads of assignments and of rows in flight
 
 // centre j = key of the (m - |P| + j)-th ranked token, a warp each; the rows up
 // to the next multiple of 16 become centres no token is near
@@ -1298,31 +1299,34 @@ __global__ void __launch_bounds__(kScatterThreads) k_lloyd_scatter(LloydArgs p) 
 // the atomics land in.  k_lloyd_finish then forms the means, one warp per
 // centre, and clears the sums for the next pass.
 //
-// The running sum of a value is a pair of floats, S from C1 = 1.5 * 2^13 and T
-// from C2 = 1.5 * 2^-4, added to without error while T's grid holds the value:
+// The running sum of a value is a pair of floats, S from C1 = 1.5 * 2^14 and T
+// from C2 = 1.5 * 2^-3, added to without error while T's grid holds the value:
 //   S' = S + x, h = S' - S, l = x - h   (Dekker's Fast2Sum, exact: |x| <= |S|)
-//   T' = T + l, g = T' - T, e = l - g   (e: what T's grid, 2^-27, drops)
+//   T' = T + l, g = T' - T, e = l - g   (e: what T's grid, 2^-26, drops)
 // so the sum is S + T - C1 - C2 exactly iff every e is zero.  S has to stay in
-// its binade [2^13, 2^14), which its exponent bits tell after every addition:
-// then |x| < 2^12 <= S, S is a multiple of 2^-10, |l| <= 2^-11, and T stays
-// within 64 * 2^-11 of C2 and is a multiple of 2^-27, so both convert to integers
-// of unit 2^-32.  Six packed fp32x2 additions and three ORs take two values
+// its binade [2^14, 2^15), which its exponent bits tell after every addition
+// (64 values below 128 always do): then |x| < 2^13 <= S, S is a multiple of 2^-9,
+// |l| <= 2^-10, and T stays within 64 * 2^-10 of C2 and is a multiple of 2^-26, so
+// both convert to integers of unit 2^-32.  Six packed fp32x2 additions and three ORs take two values
 // through it, where the integer form this replaces took 8 additions, 2 integer
 // additions and a maximum per value.
-// A value is dropped from when it is below 2^-20 in magnitude (about 8 in
+// A value is dropped from when it is below 2^-19 in magnitude (about 15 in
 // 10^7 of normally distributed values, so in a few of a unit's centres): the
-// warp then adds the exact e as 64-bit integers of unit 2^-60, kept beside and
+// warp then adds the exact e as 64-bit integers of unit 2^-59, kept beside and
 // flushed into tsum.  |e| is at most half of T's grid, 2^32 units, so the 2^30
 // members that a centre can have sum to 2^62 at most.  Sums that leave the binade
-// (64 rows that sum past 4096) or values with bits below 2^-60 flag the centre: it
-// is summed in fp64 in member order.
+// (64 rows that sum past 8192) or values with bits below 2^-59 flag the centre: it
+// is summed in fp64 in member order (k_lloyd_finish: its members are found and read
+// a few loads at a time).  C1 is the least that holds 64 values below 128 (8 units of
+// 32K keys, r = 51, a mean of 70 in one channel: 1.1 ms of iterations, with C1 = 1.5 *
+// 2^13 11.4; a mean of 300, summed in fp64, 4.9 against 5.2 a row at a time).
 constexpr int kAccRowsPerWarp = 64;
 constexpr int kAccRows = kAccRowsPerWarp * (kThreads / 32);   // member slots per CTA
-constexpr float kSumC1 = 12288.0f;
-constexpr float kSumC2 = 0x1.8p-4f;
-static_assert(kAccRowsPerWarp <= 64, "T must stay within 2^-5 of C2");
-constexpr int kTailBits = 60;                                 // unit of a dropped part: 2^-60
-constexpr float kTailScale = 0x1p60f;
+constexpr float kSumC1 = 24576.0f;
+constexpr float kSumC2 = 0x1.8p-3f;
+static_assert(kAccRowsPerWarp <= 64, "T must stay within 2^-4 of C2");
+constexpr int kTailBits = 59;                                 // unit of a dropped part: 2^-59
+constexpr float kTailScale = 0x1p59f;
 enum : uint32_t { kSumFp64 = 1u, kSumTails = 2u };            // mflag
 
 struct PairSum {
@@ -1344,7 +1348,7 @@ __device__ __forceinline__ float2 pair_add(float2 x, PairSum& a) {
 
 // The fixed-point total of one sum, unit 2^-32 (exact).
 __device__ __forceinline__ long long sum_total(float s, float t) {
-  const long long c1 = 12288ll << 32, c2 = 3ll << 27;
+  const long long c1 = 24576ll << 32, c2 = 3ll << 28;
   return (__float2ll_rz(s * 0x1p32f) - c1) + (__float2ll_rz(t * 0x1p32f) - c2);
 }
 
@@ -1544,6 +1548,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
   // members of the block's centres and their rounded reciprocals: one fp64
   // division for all of them
   __shared__ int cnt_s[kFinWarps];
+  __shared__ int mem_s[kFinWarps][32 * kFinScan + kFinRows];
   __shared__ double rcp_s[kFinWarps];
   if (threadIdx.x < kFinWarps) {
     const int jj = blockIdx.x * kFinWarps + threadIdx.x;
@@ -1588,15 +1593,17 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     }
   } else if ((flag & kSumFp64) == 0u) {
     // some values have bits below T's grid: sum = RN(S * 2^-32 + tails * 2^-kTailBits)
-    auto total = [](long long hi, long long lo) {
+    const double y = rcp_s[threadIdx.x >> 5] * 0x1p32;
+    auto mean = [&](long long hi, long long lo) {
       const __int128 v = (__int128(hi) << (kTailBits - 32)) + lo;
-      const double x = v == 0 ? 0.0 : round_u128(u128(v < 0 ? -v : v), -kTailBits, false);
-      return v < 0 ? -x : x;
+      const double a = v == 0 ? 0.0 : round_u128(u128(v < 0 ? -v : v), -kTailBits, false);
+      const double x = v < 0 ? -a : a, q0 = x * y;
+      return fma(fma(-q0, cd, x), y, q0);
     };
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      mk[q] = total(ms[32 * q], ts[32 * q]) / cd;
-      mv[q] = final_pass ? total(ms[kHeadDim + 32 * q], ts[kHeadDim + 32 * q]) / cd : 0.0;
+      mk[q] = mean(ms[32 * q], ts[32 * q]);
+      mv[q] = final_pass ? mean(ms[kHeadDim + 32 * q], ts[kHeadDim + 32 * q]) : 0.0;
     }
   } else {
     // fp64 sums over the unit's tokens in order
@@ -1605,25 +1612,49 @@ __global__ void __launch_bounds__(kFinWarps * 32) k_lloyd_finish(LloydArgs p, in
     const int32_t* as = p.assign + int64_t(u) * p.s;
     const __nv_bfloat16* Kd = p.K + int64_t(ul) * p.s * kHeadDim + 4 * lane;
     const __nv_bfloat16* Vd = p.V + int64_t(ul) * p.s * kHeadDim + 4 * lane;
-    for (int64_t t0 = 0; t0 < p.s; t0 += 32) {
-      unsigned take = __ballot_sync(0xffffffffu, t0 + lane < p.s && as[t0 + lane] == j);
-      for (; take != 0u; take &= take - 1) {
-        const int64_t pos = t0 + __ffs(take) - 1;
-        const uint2 kw = *reinterpret_cast<const uint2*>(Kd + pos * kHeadDim);
-        const float2 k01 = bf16x2_to_float2(kw.x), k23 = bf16x2_to_float2(kw.y);
-        tk[0] += double(k01.x);
-        tk[1] += double(k01.y);
-        tk[2] += double(k23.x);
-        tk[3] += double(k23.y);
-        if (final_pass) {
-          const uint2 vw = *reinterpret_cast<const uint2*>(Vd + pos * kHeadDim);
-          const float2 v01 = bf16x2_to_float2(vw.x), v23 = bf16x2_to_float2(vw.y);
-          tv[0] += double(v01.x);
-          tv[1] += double(v01.y);
-          tv[2] += double(v23.x);
-          tv[3] += double(v23.y);
+    int* mem = mem_s[threadIdx.x >> 5];           // members found and not yet added
+    int found = 0;
+    // rows mem[i .. i + kFinRows - 1] of X (below n) into t
+    auto add_rows = [&](const __nv_bfloat16* X, int i, int n, double (&t)[4]) {
+      uint2 w[kFinRows];
+#pragma unroll
+      for (int q = 0; q < kFinRows; ++q)
+        if (i + q < n) w[q] = __ldg(reinterpret_cast<const uint2*>(X + int64_t(mem[i + q]) * kHeadDim));
+#pragma unroll
+      for (int q = 0; q < kFinRows; ++q)
+        if (i + q < n) {
+          const float2 a = bf16x2_to_float2(w[q].x), b = bf16x2_to_float2(w[q].y);
+          t[0] += double(a.x);
+          t[1] += double(a.y);
+          t[2] += double(b.x);
+          t[3] += double(b.y);
         }
+    };
+    for (int64_t t0 = 0; t0 < p.s; t0 += 32 * kFinScan) {
+      int a[kFinScan];
+#pragma unroll
+      for (int k = 0; k < kFinScan; ++k) {
+        const int64_t pos = t0 + 32 * k + lane;
+        a[k] = pos < p.s ? __ldg(as + pos) : -1;
       }
+#pragma unroll
+      for (int k = 0; k < kFinScan; ++k) {
+        const unsigned take = __ballot_sync(0xffffffffu, a[k] == j);
+        if (a[k] == j) mem[found + __popc(take & ((1u << lane) - 1u))] = int(t0) + 32 * k + lane;
+        found += __popc(take);
+      }
+      __syncwarp();
+      const int n = t0 + 32 * kFinScan < p.s ? found & ~(kFinRows - 1) : found;
+      for (int i = 0; i < n; i += kFinRows) {
+        add_rows(Kd, i, n, tk);
+        if (final_pass) add_rows(Vd, i, n, tv);
+      }
+      // (fewer than kFinRows left)
+      const int left = lane < found - n ? mem[n + lane] : 0;
+      __syncwarp();
+      if (lane < found - n) mem[lane] = left;
+      found -= n;
+      __syncwarp();
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
