@@ -176,6 +176,10 @@ typedef struct reskv_cache reskv_cache;
  *                              residual_override set
  *   out                      : receives a new handle on success
  *
+ * Alignment (RESKV_ERR_INVALID_ARG otherwise): Qobs 4 bytes; V 8 bytes, 16 with
+ * the validation proxy; K 16 bytes, or 8 with RESKV_SCORE_KEYNORM and no proxy
+ * where no residual entry is asked for or a layer has fewer than 128 keys.
+ *
  * Inputs may be freed once the stream has passed the call.  The call
  * allocates the handle's device memory (cudaMalloc) and temporary workspace.
  */

@@ -281,6 +281,19 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
   for (int32_t r : col_rmax) rmax = std::max(rmax, r);
   if (rmax > kMaxR) return fail(RESKV_ERR_UNSUPPORTED, "residual entries per unit must be <= 8192");
   const int rstride = (rmax + 15) & ~15;             // stride of the per-centre arrays
+  // What the kernels read at once: whole key tiles and 16-byte chunks for
+  // observation scores, the assignment (tiles of 128 keys by TMA; fewer keys are
+  // copied) and the proxy, whose losses take the values the same way; else rows in
+  // 8-byte pieces.  Queries come in 4-byte words.
+  const uintptr_t k_align = cfg.score_mode == RESKV_SCORE_OBS_POOL || proxy ||
+                            (rmax > 0 && int64_t(UL) * s >= kTile) ? 16 : 8;
+  const uintptr_t v_align = proxy ? 16 : 8;
+  auto aligned = [](const void* p, uintptr_t to) { return reinterpret_cast<uintptr_t>(p) % to == 0; };
+  for (int l = 0; l < cfg.n_layers; ++l)
+    if (!aligned(Kl[l], k_align) || !aligned(Vl[l], v_align) || (need_q && !aligned(Ql[l], 4)))
+      return fail(RESKV_ERR_INVALID_ARG,
+                  "layer " + std::to_string(l) + ": K must be " + std::to_string(k_align) + "-byte aligned, V " +
+                      std::to_string(v_align) + "-byte, Qobs 4-byte");
 
   // ---------------- handle and scratch ----------------
   reskv_cache* c = nullptr;
