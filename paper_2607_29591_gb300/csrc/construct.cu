@@ -565,7 +565,6 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       return cleanup_fail(fail(RESKV_ERR_CUDA, "launching the ranking"));
     RESKV_LAUNCH_CHECK("ranking");
     // candidate r per unit of this layer
-    int grid_r = rmax;
     if (proxy) {
       if (per_unit || l == 0) unit_candidates(bl_h, hr);
       for (int c2 = 1; c2 < ncol; ++c2)
@@ -574,8 +573,6 @@ reskv_status build_all_layers(reskv_cache** out, const reskv_config& cfg,
       if ((per_unit || l == 0) &&
           cudaMemcpyAsync(r_runs, hr.data(), hr.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess)
         return cleanup_fail(fail(RESKV_ERR_CUDA, "copying candidate budgets"));
-      grid_r = 0;
-      for (int32_t r : hr) grid_r = std::max<int>(grid_r, r);
     }
 
     LloydArgs la{};

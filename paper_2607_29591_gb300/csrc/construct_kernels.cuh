@@ -154,14 +154,11 @@ __device__ __forceinline__ void obs_logits(uint32_t ks_s, int tk, int lane, cons
 }
 
 // Warps of a block of the first pass: one per pair of row blocks where there are
-// few, else the count of 4, 3 or 6 that leaves the fewest idle in the last round.
+// few, else 4, or 3 where that leaves fewer idle in the last round.
 __host__ inline int obs_warps1(int n_rows) {
   const int pairs = ((n_rows + 15) / 16 + 1) / 2;
   if (pairs <= 3) return pairs;
-  int best = 4;
-  for (int w : {3, 6})
-    if ((pairs + w - 1) / w * w < (pairs + best - 1) / best * best) best = w;
-  return best;
+  return (pairs + 2) / 3 * 3 < (pairs + 3) / 4 * 4 ? 3 : 4;
 }
 // of the second: its items are (pair of partial sums, half of the tile)
 __host__ inline int obs_warps2(int n_rows) {
@@ -199,7 +196,7 @@ __device__ __forceinline__ void obs_fold(const float (&S)[8][4], int a, int t4, 
 }
 
 // Pass 1: per (row, tile) max and sum of 2^{a log2e} over the tile's tokens.
-__global__ void __launch_bounds__(192, 2) k_obs_pass1(ObsArgs p) {
+__global__ void __launch_bounds__(128, 3) k_obs_pass1(ObsArgs p) {
   extern __shared__ __align__(128) uint8_t obs_raw[];
   const int tile = blockIdx.x, ul = blockIdx.y;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
