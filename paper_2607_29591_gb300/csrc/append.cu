@@ -37,7 +37,9 @@
 // dependent loads: the counts, the rows, the chosen entry.  One CTA of 8 warps
 // per unit keeps 64 rows in flight; the launch is a programmatic dependent
 // launch, and everything up to the new token's rows is read before the wait
-// for the previous kernel, which is a decode that only reads the cache.
+// for the previous kernel, which is a decode that only reads the cache.  (On the
+// SMs the decode leaves free: a CTA of 98 registers x 256 threads does not fit
+// beside one of the cluster decode's 200 x 256.)
 // Measured on 64 units a layer with 0..204 entries (32K, b = 1024, B = 8), an
 // append and a decode per layer: 17.3 us a layer, of which the decode alone
 // takes 7.9; 244 us before, when one warp per unit took the 128-bit sums over

@@ -29,8 +29,8 @@ reskv_status fail(reskv_status st, const std::string& msg) {
 }
 
 // The construction's scratch arrays, in one device allocation: every cudaMalloc
-// and cudaFree costs 10 to 40 us of host time beside its kernels (a build of 8
-// units of 32K keys spent 1.4 of its 5.3 ms on 37 pairs of them).  get() places
+// and cudaFree costs 10 us of host time beside its kernels, up to 700 for 1 GB (a
+// build of 8 units of 32K keys spent 1.4 of its 5.3 ms on 37 pairs of them).  get() places
 // an array, commit() allocates and sets every pointer.
 class Scratch {
  public:

@@ -98,7 +98,9 @@ struct ObsArgs {
 // blocks per SM cover each other's loads.  64 units of 32K keys, 96 rows: passes
 // 361 + 472 us -> 204 + 252; 32 units of 128K keys, 384 rows: 2039 + 2579 ->
 // 1375 + 1273 (the tensor pipe, busy for about half of that, and the issue of the
-// exponentials between the products bound it now).
+// exponentials between the products bound it now; the second pass, at 168
+// registers, spills 228 bytes a thread and reads 396 back: two blocks per SM
+// without the spills took 350 us where this takes 252).
 __global__ void k_obs_frag(ObsArgs p) {          // grid (blocks of rows, UL), 256 threads
   const int rb = blockIdx.x, ul = blockIdx.y;
   const int ks = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;

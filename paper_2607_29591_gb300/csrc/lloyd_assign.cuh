@@ -10,7 +10,7 @@
 //
 // k_lloyd_assign: a persistent CTA per SM walks a contiguous range of (unit,
 // tile) pairs with the unit's planes resident in shared memory, so a tile costs
-// one key-tile load and one MMA chain.  Three roles, linked by mbarriers:
+// one key-tile load and one MMA chain.  Four roles, linked by mbarriers:
 //
 //   loader warp      key tiles by TMA (both 64-dim halves, 128-byte swizzle,
 //                    one 32 KB copy) into a ring of nk buffers, and the tokens'
@@ -36,10 +36,10 @@
 //   4 deciders       join the four column quarters' candidates of 32 tokens each
 //                    and decide.
 //
-// W is a rigorous bound on what rounding can have moved, so a centre outside it
-// cannot be nearest.  A token left with one centre is decided; the others (a few
-// per cent) join a list of the CTA that k_lloyd_resolve decides exactly.  The two
-// sweeps take 1.5 integer-pipe operations per distance, where a running best
+// W bounds what rounding can have moved (below), so a centre outside it cannot be
+// nearest.  A token left with one centre is decided; the others (less than one per
+// cent of centred keys) join a list of the CTA that k_lloyd_resolve decides exactly.
+// The two sweeps take 1.5 integer-pipe operations per distance, where a running best
 // three with packed indices took 6 and bounded the assignment.
 //
 // Units with more than 256 centres take their centres in segments of at most
@@ -62,14 +62,17 @@
 // 17 * 2^-22 times the largest partial magnitude (<= P) even if it truncates to
 // 24 bits; 16 chained steps (both planes) give 272 * 2^-22 P = 1088u P, the split
 // e adds 256u P, |c1| + |c2| exceeds |c| by 2^-8: 1350u P, taken as 1440u P.  (A
-// bound three times as wide cost k_lloyd_resolve 1.7 to 2.1 times its time.)
+// bound three times as wide cost k_lloyd_resolve 1.7 to 2.1 times its time.  Measured
+// on GB300 over 43 kinds of rows -- one sign, one product far above the others in a
+// step or in the chain, cancelling ones, every alignment to the accumulator -- a chain
+// was never more than 45u P off where 1088u P is allowed.)
 // Values, products and sums below 2^-126 may be lost besides, whole at worst: 2^-126
 // sum_i (|c_i| + |k_i|) <= 12 * 2^-126 (||c|| + ||k||) for the operands, twice that in a
 // distance, and some 600 terms of 2^-126.  So W is positive however small the
 // distances are, and centres at equal ones (all of them zero, say) are candidates.
 //
 // What bounds it: issue and the latency of a tile's steps (about 2.3 instructions
-// per cycle; the tensor pipe is active 28 % of the time at r = 51 and 54 % at 204,
+// per cycle; the tensor pipe is active 27 % of the time at r = 51 and 54 % at 204,
 // DRAM 66 % and 41 %).  64 units of 32K keys (16384 tiles) take 108, 125, 150 and
 // 178 us at r = 51, 102, 153, 204; the running best three took 148, 180, 221 and
 // 265.  32 units of 128K keys at r = 409 take 685 us in two segments, where a
@@ -119,8 +122,8 @@ constexpr long long kTcWaitCycles = 4000000000LL;
 // Dynamic shared memory, from a 1024-aligned base: the planes of rp = r rounded
 // up to 16 centres ([plane][64-dim half][rp rows][128 B], 512 rp bytes) and nk
 // key tiles of 32 KB.  The small parts are static, so that their addresses cost
-// no registers: the column warps hold 64 distances in the 96 registers that 18
-// warps leave them, and what spilled would not fit the L1 beside 220 KB.
+// no registers: the column warps hold 64 distances in their 88 registers
+// (kAsgRegsCol), and what spilled would not fit the L1 beside 220 KB.
 struct AsgShared {
   float cn[2][kAsgRmax];                               // centre norms (two units)
   int2 xch[2][4][kTile];                               // the column quarters' candidates (two tiles)
