@@ -538,9 +538,9 @@ __device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
 
 // 128 fp32 products summed in any order stay within 130 u of the sum, the root
 // and the product within 2 u each; what underflows is below 255 * 2^-150, its root
-// below kNormLost
-constexpr float kNormLost = 0x1p-70f;
-__device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.0f + 140.0f * 5.9604645e-8f) + kNormLost; }
+// far below kNormLost, which the caller adds (2^-50: see k_lloyd_assign's bound)
+constexpr float kNormLost = 0x1p-50f;
+__device__ __forceinline__ float norm_bound(float sum) { return sqrtf(sum) * (1.0f + 140.0f * 5.9604645e-8f); }
 
 // Per key row, in one read of the keys: with kScore the query-free score, and
 // (knorm not NULL) an upper bound of ||k|| for the Lloyd assignment's rounding
@@ -652,14 +652,14 @@ __global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restri
     }
   }
   if constexpr (!kScore) {
-    if (mine < n_rows) knorm[mine] = norm_bound(fsum);
+    if (mine < n_rows) knorm[mine] = norm_bound(fsum) + kNormLost;
   } else {
     if (mine < n_rows && e0) {
       scores[mine] = __ull2double_rn(sum) * __hiloint2double((1023 + 2 * (e0 - 134)) << 20, 0);
       if (knorm) {
         const int E = e0 - 134;
         const float unit = __uint_as_float(E >= -126 ? uint32_t(E + 127) << 23 : 1u << (E + 149));
-        const float nrm = __fmul_ru(norm_bound(__ull2float_ru(sum)), unit);
+        const float nrm = __fmul_ru(norm_bound(__ull2float_ru(sum)), unit) + kNormLost;
         knorm[mine] = nrm < 1.8446744e19f ? nrm : INFINITY;        // as the fp32 sum: beyond 2^64 no bound
       }
     }
@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(256) k_key_norms(const __nv_bfloat16* __restri
       const float f = warp_sum(fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, b.y * b.y))));
       if (lane == 0) {
         scores[row] = sc;
-        if (knorm) knorm[row] = norm_bound(f);
+        if (knorm) knorm[row] = norm_bound(f) + kNormLost;
       }
     }
   }

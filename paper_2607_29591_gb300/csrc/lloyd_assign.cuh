@@ -68,8 +68,10 @@
 // was never more than 45u P off where 1088u P is allowed.)
 // Values, products and sums below 2^-126 may be lost besides, whole at worst: 2^-126
 // sum_i (|c_i| + |k_i|) <= 12 * 2^-126 (||c|| + ||k||) for the operands, twice that in a
-// distance, and some 600 terms of 2^-126.  So W is positive however small the
-// distances are, and centres at equal ones (all of them zero, say) are candidates.
+// distance, and some 600 terms of 2^-126.  The bounds of both norms are kNormLost =
+// 2^-50 above them, which adds 2^-62 (||c|| + ||k||) + 2^-112 to W's dot products: more
+// than all of that.  So W is positive however small the distances are, and centres
+// at equal ones (all of them zero, say) are candidates.
 //
 // What bounds it: issue and the latency of a tile's steps (about 2.3 instructions
 // per cycle; the tensor pipe is active 27 % of the time at r = 51 and 54 % at 204,
@@ -415,11 +417,11 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
       const float d0 = fminf(min3(a[0], a[1], a[2]), a[3]);
       // A computed distance is off by at most ee + 4u |d| from the exact distance
       // to the fp64 centre: ee = 2 x dot product (gam_tc ||c|| ||k||, and 2u for
-      // the fp32 centre) + norm sum gam ||c||^2 (130u, and 2u for the fp32 centre)
-      // + what underflows, ||c|| <= max ||c|| over the unit.  So the nearest
-      // centre's computed distance is within 2 ee + 4u (|d0| + |d|) of d0.
+      // the fp32 centre) + norm sum gam ||c||^2 (130u, and 2u for the fp32 centre),
+      // ||c|| <= max ||c|| over the unit.  So the nearest centre's computed
+      // distance is within 2 ee + 4u (|d0| + |d|) of d0.
       const float uu = 5.9604645e-8f, gam = 140.0f * uu, gam_tc = 1440.0f * uu;
-      const float ee = fmaf(cm, 2.0f * gam_tc * kn + gam * cm, fmaf(0x1p-121f, kn + cm, 0x1p-116f));
+      const float ee = cm * (2.0f * gam_tc * kn + gam * cm);
       const float ww = 2.01f * ee;
       const float thr = d0 + asg_window(ww, d0);
       const float2 nthr = make_float2(-thr, -thr);
@@ -437,13 +439,8 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
         const uint32_t v = (((w[0] << 4) | w[1]) << 8) | (w[2] << 4) | w[3];
         m[i >> 1] |= (i & 1) ? v : v << 16;
       }
-      // Below a window of 1e32 every product, sum and norm is finite.  Past it a
-      // centre may lie beside the token at a distance that overflowed, so all
-      // centres are candidates (where any distance is a number at all).
-      AsgCand cd{d0, 0, 0, ww < 1e32f ? min(__popc(m[0]) + __popc(m[1]), 3) : d0 < INFINITY ? 3 : 0};
-      if (cd.n == 0) {                                    // no centre, or NaN or infinite distances
-        cd.d = INFINITY;
-      } else {
+      AsgCand cd{d0, 0, 0, min(__popc(m[0]) + __popc(m[1]), 3)};
+      if (cd.n != 0) {                                    // (else no centre, or NaN or infinite distances)
         const int pf = m[0] != 0u ? __clz(m[0]) : 32 + __clz(m[1]);
         const int pl = m[1] != 0u ? 64 - __ffs(m[1]) : 32 - __ffs(m[0]);
         cd.first = seg0 + 16 * quarter + (pf & 15) + ((pf & 48) << 2);
@@ -644,6 +641,13 @@ __global__ void __launch_bounds__(kAsgThreads, 1)
         AsgCand cd = join(AsgCand::unpack(x0), AsgCand::unpack(x1));
         cd = join(cd, AsgCand::unpack(x2));
         cd = join(cd, AsgCand::unpack(x3));
+        // Below a window of 1e32 every product, sum and norm is finite.  Past it a
+        // centre may lie beside the token at a distance that overflowed, so all
+        // centres are candidates (where any distance is a number below infinity).
+        if (!(ww < 1e32f)) {
+          const float d = fminf(min3(__int_as_float(x0.x), __int_as_float(x1.x), __int_as_float(x2.x)), __int_as_float(x3.x));
+          cd = AsgCand{d, 0, 0, d < INFINITY ? 3 : 0};
+        }
         if (seg0 > 0 && mine) cd = join(AsgCand::unpack(p.cand[tix]), cd);   // the segments before
         if (r > seg0 + segw) {                              // more centres in the next launch
           if (mine) p.cand[tix] = cd.pack();
