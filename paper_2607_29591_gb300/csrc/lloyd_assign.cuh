@@ -75,7 +75,7 @@
 //
 // What bounds it: issue and the latency of a tile's steps (about 2.3 instructions
 // per cycle; the tensor pipe is active 27 % of the time at r = 51 and 54 % at 204,
-// DRAM 66 % and 41 %).  64 units of 32K keys (16384 tiles) take 108, 129, 149 and
+// DRAM 66 % and 41 %).  64 units of 32K keys (16384 tiles) take 112, 129, 149 and
 // 177 us at r = 51, 102, 153, 204; the running best three took 148, 180, 221 and
 // 265.  32 units of 128K keys at r = 409 take 685 us in two segments, where a
 // kernel that streamed the centres per tile took 4500.
